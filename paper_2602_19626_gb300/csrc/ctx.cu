@@ -50,6 +50,8 @@ struct Slot {
 constexpr int kPfBuckets = 4;
 struct TcMat {
   CUtensorMap a;
+  CUtensorMap a_dec, b_dec;          // a decode step's maps: 2D, boxes of 32 rows
+  int dec_pro = -1;                  // how its operand is made there (DecPro), -1: not used
   CUtensorMap b[2][4];               // per forward buffer set
   int M = 0, K = 0;
   int kp = 1;                        // 2: 3D maps, two K blocks per pipeline stage (TcGemm::kp)
@@ -541,6 +543,16 @@ static int tc_setup(nc_ctx* ctx) {
     for (int bi = 0; bi < 4; ++bi)
       if (!tc_encode_operand(t, &t.b[0][bi], src, esz, R, 32 << bi))
         return fail(ctx, NC_ECUDA, "tensor map encoding failed");
+    if (q < 4) {
+      const int pro = (q == 0 || q == 2) ? DPRO_RMS : kb ? DPRO_TMA : DPRO_FP8;
+      if (gemm_dec_fits(kb, t.K, pro)) {
+        t.dec_pro = pro;
+        const void* w = q == 0 ? ctx->layers[i / 4].qkv.w : q == 1 ? ctx->layers[i / 4].o.w
+                        : q == 2 ? ctx->layers[i / 4].gu.w : ctx->layers[i / 4].down.w;
+        if (!tc_encode_tmap(&t.a_dec, w, esz, t.K, t.M, 32) || !tc_encode_tmap(&t.b_dec, src, esz, t.K, R, 32))
+          return fail(ctx, NC_ECUDA, "tensor map encoding failed");
+      }
+    }
     if (ctx->n_fs == 2) {
       const void* src1 = (kb && q == 3) ? ctx->fs[1].opnd2 : ctx->fs[1].opnd;
       for (int bi = 0; bi < 4; ++bi)
@@ -754,7 +766,7 @@ extern "C" int nc_ctx_create(const nc_config* cfg, const void* weights, size_t n
   if (cudaMemset(ctx->d_st, 0, B * sizeof(StreamDev)) != cudaSuccess) return bail(NC_ECUDA);
   if (cudaMemset(ctx->d_status, 0, B * 4) != cudaSuccess) return bail(NC_ECUDA);
   if (prepare_model_kernels(D, ctx->fmt) != cudaSuccess || prepare_vocab_kernels(D) != cudaSuccess ||
-      (c.path == NC_PATH_TC && prepare_tc_kernels() != cudaSuccess))
+      (c.path == NC_PATH_TC && (prepare_tc_kernels() != cudaSuccess || prepare_dec_kernels() != cudaSuccess)))
     return bail(NC_ECUDA);
   if (c.path == NC_PATH_TC) {
     const int st2 = tc_setup(ctx);
@@ -1043,28 +1055,65 @@ static cudaError_t launch_model_tc(nc_ctx* ctx, const Batch& b, StepMarks& m, in
     g.status = ctx->d_status;
     return launch_gemm_tc(g, epi, s, D.pdl);
   };
+  // a decode step of a few rows: the projections that make their own operand
+  const bool few = !b.pos && set == 0 && b.Bmax <= kDecMaxRows;
+  auto own = [&](const TcMat& t) { return few && t.dec_pro >= 0; };
+  auto gemm_dec = [&](const TcMat& t, int epi, const float* x, const float* gain, float* y, void* h16 = nullptr) {
+    TcDec g{};
+    g.tmap_a = &t.a_dec;
+    g.tmap_b = t.dec_pro == DPRO_TMA ? &t.b_dec : nullptr;
+    g.M = t.M;
+    g.K = t.K;
+    g.Bmax = b.Bmax;
+    g.nB = b.nB;
+    g.x = x;
+    g.gain = gain;
+    g.eps = D.eps;
+    g.w_scale = t.scale;
+    if (epi == EPI_SWIGLU) g.h_out = y;
+    else g.y = y;
+    g.h16 = h16;
+    g.status = ctx->d_status;
+    return launch_gemm_dec(g, kb, epi, t.dec_pro, s, D.pdl);
+  };
   cudaError_t e = launch_embed(D, b, ctx->embed, ctx->embed_scale, ctx->fmt, F.x, s);
   if (e == cudaSuccess) e = m.mark(s, TK_EMBED);
   for (int l = 0; l < D.n_layers && e == cudaSuccess; ++l) {
     const LayerW& L = ctx->layers[l];
     const TcMat* T = &ctx->tc[4 * l];
-    e = launch_act_rmsnorm(D, b, F.x, L.g_attn, D.d, kb, F.opnd, F.opnd_scale, s);
-    if (e == cudaSuccess) e = gemm(T[0], EPI_STORE, F.qkv, nullptr);
+    if (own(T[0])) {
+      e = gemm_dec(T[0], EPI_STORE, F.x, L.g_attn, F.qkv);
+    } else {
+      e = launch_act_rmsnorm(D, b, F.x, L.g_attn, D.d, kb, F.opnd, F.opnd_scale, s);
+      if (e == cudaSuccess) e = gemm(T[0], EPI_STORE, F.qkv, nullptr);
+    }
     if (e == cudaSuccess && b.pos && sync.wait) e = cudaStreamWaitEvent(s, sync.wait[l], 0);
     if (e == cudaSuccess && b.pos) e = launch_kv_append(D, b, l, F.qkv, s);
     if (e == cudaSuccess) e = m.mark(s, TK_QKV);
     if (e == cudaSuccess) e = launch_attn(D, b, l, F.qkv, F.attn_out, s, kb ? F.opnd : nullptr);
     if (e == cudaSuccess && sync.rec) e = cudaEventRecord(sync.rec[l], s);
     if (e == cudaSuccess) e = m.mark(s, TK_ATTN);
-    if (e == cudaSuccess && !kb)
-      e = launch_act_plain(D, b, F.attn_out, D.hq * kHeadDim, kb, F.opnd, F.opnd_scale, s);
-    if (e == cudaSuccess) e = gemm(T[1], EPI_RESID, F.x, nullptr);
+    if (e == cudaSuccess && own(T[1])) {
+      e = gemm_dec(T[1], EPI_RESID, F.attn_out, nullptr, F.x);
+    } else {
+      if (e == cudaSuccess && !kb)
+        e = launch_act_plain(D, b, F.attn_out, D.hq * kHeadDim, kb, F.opnd, F.opnd_scale, s);
+      if (e == cudaSuccess) e = gemm(T[1], EPI_RESID, F.x, nullptr);
+    }
     if (e == cudaSuccess) e = m.mark(s, TK_O);
-    if (e == cudaSuccess) e = launch_act_rmsnorm(D, b, F.x, L.g_ffn, D.d, kb, F.opnd, F.opnd_scale, s);
-    if (e == cudaSuccess) e = gemm(T[2], EPI_SWIGLU, nullptr, F.h, kb ? F.opnd2 : nullptr);
+    if (e == cudaSuccess && own(T[2])) {
+      e = gemm_dec(T[2], EPI_SWIGLU, F.x, L.g_ffn, F.h, kb ? F.opnd2 : nullptr);
+    } else {
+      if (e == cudaSuccess) e = launch_act_rmsnorm(D, b, F.x, L.g_ffn, D.d, kb, F.opnd, F.opnd_scale, s);
+      if (e == cudaSuccess) e = gemm(T[2], EPI_SWIGLU, nullptr, F.h, kb ? F.opnd2 : nullptr);
+    }
     if (e == cudaSuccess) e = m.mark(s, TK_GU);
-    if (e == cudaSuccess && !kb) e = launch_act_plain(D, b, F.h, D.F, kb, F.opnd, F.opnd_scale, s);
-    if (e == cudaSuccess) e = gemm(T[3], EPI_RESID, F.x, nullptr);
+    if (e == cudaSuccess && own(T[3])) {
+      e = gemm_dec(T[3], EPI_RESID, F.h, nullptr, F.x);
+    } else {
+      if (e == cudaSuccess && !kb) e = launch_act_plain(D, b, F.h, D.F, kb, F.opnd, F.opnd_scale, s);
+      if (e == cudaSuccess) e = gemm(T[3], EPI_RESID, F.x, nullptr);
+    }
     if (e == cudaSuccess) e = m.mark(s, TK_DOWN);
   }
   if (e == cudaSuccess) e = launch_act_rmsnorm(D, b, F.x, ctx->g_final, D.d, kb, F.opnd, F.opnd_scale, s);

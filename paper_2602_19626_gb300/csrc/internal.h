@@ -170,7 +170,10 @@ __device__ __forceinline__ size_t kv_plane_off(int L, int hkv, int layer, int wh
 // no in-flight kernel writes (weights, KV entries of earlier tokens, state of
 // earlier steps) before pdl_wait(), and signals its own dependents only
 // after pdl_wait(); so when a kernel's pdl_wait() returns, every earlier
-// kernel of the stream has completed and its writes are visible.
+// kernel of the stream has completed and its writes are visible.  (Signalling
+// before the wait too, so that several kernels' weights are in flight, was
+// tried on the decode step: 907 us a token against 854, the waiting CTAs'
+// traffic slowed the running kernel more than it hid.)
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -317,6 +320,31 @@ struct TcGemm {
   const int32_t* slots;
   int32_t* status;          // error word (ST_TIMEOUT)
 };
+// The projection of a decode step of at most kDecMaxRows rows (k_gemm_dec.cu):
+// the same products in the same order, with the operand made in the kernel.
+// The line is the row tile of its norm prologue: past 64 rows every CTA would
+// make more rows than the row kernel spreads over the whole chip.
+enum DecPro { DPRO_TMA = 0, DPRO_RMS = 1, DPRO_FP8 = 2 };   // operand: by TMA, RMSNorm of x, E4M3 of x
+constexpr int kPlainVecs = 12;              // DPRO_FP8: float4 values of a row per lane (1,536 columns)
+constexpr int kDecSmemMax = 227 * 1024;
+constexpr int kDecMaxRows = 64;
+struct TcDec {
+  const void* tmap_a;       // host copy of the weights' CUtensorMap (2D, box 32 rows)
+  const void* tmap_b;       // DPRO_TMA: the operand's (2D, box 32 rows), else nullptr
+  int M, K, Bmax;
+  const int32_t* nB;
+  const float* x;           // DPRO_RMS / DPRO_FP8: FP32 rows [Bmax][K]
+  const float* gain;        // DPRO_RMS
+  float eps;
+  const float* w_scale;     // FP8: [M]
+  float* y;                 // EPI_STORE / EPI_RESID: [Bmax][M]
+  float* h_out;             // EPI_SWIGLU: [Bmax][M / 2], or
+  void* h16;                // rounded to BF16 there
+  int32_t* status;
+};
+bool gemm_dec_fits(int kind_bf16, int K, int pro);
+cudaError_t prepare_dec_kernels();
+cudaError_t launch_gemm_dec(const TcDec& g, int kind_bf16, int epi, int pro, cudaStream_t s, bool pdl);
 bool tc_encode_tmap(void* tmap, const void* base, int elem_bytes, int64_t inner, int64_t outer, int box_outer);
 bool tc_encode_tmap3(void* tmap, const void* base, int elem_bytes, int64_t K, int64_t rows, int box_rows);
 cudaError_t launch_gemm_tc(const TcGemm& g, int epi, cudaStream_t s, bool pdl);

@@ -441,19 +441,24 @@ __global__ void __launch_bounds__(kT5Threads, 2) k_attn_t5(Dims D, Batch b, int 
     // the queries, the copied rows and every K box are in place
     ok = __syncthreads_and(my_ok && mbar_wait(bar_k, 0));
     fence_after_sync();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = uniform(*tmem_slot);
+    const int warp = uniform_warp();
+    const uint64_t dq = sdesc_sw128(uniform(smem_u32(qt))), dk = sdesc_sw128(uniform(smem_u32(kt))),
+                   dv = sdesc_sw128_mn(uniform(smem_u32(vt)));
     const uint32_t tlane = tmem + ((uint32_t)(32 * ((tid >> 5) & 3)) << 16);
-    if (tid == 0 && ok) {
-      const uint32_t ids = idesc(1, kT5Pairs, kT5Block);
-      for (int bb = 0; bb < nblk; ++bb) {
+    if (warp == 0 && ok) {
+      if (elect_one()) {
+        const uint32_t ids = idesc(1, kT5Pairs, kT5Block);
+        for (int bb = 0; bb < nblk; ++bb) {
 #pragma unroll
-        for (int k = 0; k < kHeadDim / 16; ++k)
-          mma_issue(1, tmem + kT5Block * bb, sdesc_sw128(smem_u32(qt) + 32 * k),
-                    sdesc_sw128(smem_u32(kt + bb * kT5Block * kRowB) + 32 * k), ids, k ? 1u : 0u);
+          for (int k = 0; k < kHeadDim / 16; ++k)   // descriptor addresses count 16 bytes
+            mma_issue(1, tmem + kT5Block * bb, dq + 2 * k, dk + (uint64_t)(bb * (kT5Block * kRowB / 16) + 2 * k), ids,
+                      k ? 1u : 0u);
+        }
+        mma_commit(bar_s);
       }
-      mma_commit(bar_s);
+      __syncwarp();
     }
-    __syncwarp();
     // every score product done (the key and query tiles hold the P buffers
     // from here) and every V box in place
     ok = __syncthreads_and(ok && mbar_wait(bar_s, 0) && mbar_wait(bar_v, 0));
@@ -492,19 +497,21 @@ __global__ void __launch_bounds__(kT5Threads, 2) k_attn_t5(Dims D, Batch b, int 
       fence_before_sync();
       ok = __syncthreads_and(ok && wok);
       fence_after_sync();
-      if (tid == 0 && ok && 2 * k < nblk) {
+      if (warp == 0 && ok && 2 * k < nblk) {
         // O_c += P_b V_b for the stage's blocks, into columns 0 .. 63
-        const uint32_t ido = idesc(1, kT5Pairs, kHeadDim, 1);
-        for (int b2 = 2 * k; b2 < min(2 * k + 2, nblk); ++b2) {
-          uint8_t* pt2 = b2 == 2 ? qt : kt + (b2 & 1) * (kT5Pairs * kRowB);
+        if (elect_one()) {
+          const uint32_t ido = idesc(1, kT5Pairs, kHeadDim, 1);
+          for (int b2 = 2 * k; b2 < min(2 * k + 2, nblk); ++b2) {
+            const uint64_t dp = b2 == 2 ? dq : dk + (uint64_t)((b2 & 1) * (kT5Pairs * kRowB / 16));
 #pragma unroll
-          for (int s = 0; s < kT5Block / 16; ++s)
-            mma_issue(1, tmem, sdesc_sw128(smem_u32(pt2) + 32 * s),
-                      sdesc_sw128_mn(smem_u32(vt + (b2 * kT5Block + 16 * s) * kRowB)), ido, b2 + s ? 1u : 0u);
+            for (int s = 0; s < kT5Block / 16; ++s)
+              mma_issue(1, tmem, dp + 2 * s, dv + (uint64_t)((b2 * kT5Block + 16 * s) * (kRowB / 16)), ido,
+                        b2 + s ? 1u : 0u);
+          }
+          mma_commit(k ? bar_o1 : bar_o0);
         }
-        mma_commit(k ? bar_o1 : bar_o0);
+        __syncwarp();
       }
-      __syncwarp();
     }
     red[wg * kT5Pairs + p] = lh;
     // every product done
@@ -532,7 +539,7 @@ __global__ void __launch_bounds__(kT5Threads, 2) k_attn_t5(Dims D, Batch b, int 
     // give-up path: every copy and product issued has completed before the
     // memory is freed
     if (!ok) {
-      if (tid == 0) mma_commit(bar_done);
+      if (warp == 0 && elect_one()) mma_commit(bar_done);
       __syncwarp();
       mbar_wait(bar_done, 0);
       mbar_wait(bar_k, 0);

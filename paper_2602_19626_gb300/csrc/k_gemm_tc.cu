@@ -23,6 +23,7 @@
 
 #include "internal.h"
 #include "tc5.cuh"
+#include "tc_row.cuh"
 
 namespace nc {
 
@@ -33,11 +34,6 @@ using namespace tc5;
 constexpr int kTcThreads = 256;              // 8 warps: all read the accumulator back
 constexpr int kTileM = 128;
 constexpr int kKBlockBytes = 128;            // one 128-byte swizzle row per operand row
-// SiLU of the tensor-core path: a * (1 / (1 + e^-a)) with the fast exponential
-// and a correctly rounded reciprocal (1 / inf = 0 for very negative a).  The
-// decode step and the prefill forward run this same code.
-__device__ __forceinline__ float silu_tc(float a) { return a * __frcp_rn(1.0f + __expf(-a)); }
-
 template <int BN>
 __host__ __device__ constexpr uint32_t tmem_cols() {
   return BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;
@@ -48,24 +44,6 @@ __host__ __device__ constexpr size_t tc_smem_bytes() {
   return 1024 /* alignment slack */ + (size_t)STAGES * KP * (kTileM + BN) * kKBlockBytes + 256;
 }
 
-// SwiGLU of two adjacent batch columns n, n + 1: rows 2j (gate) and 2j + 1
-// (up) sit on adjacent lanes; the even lane computes h_j of column n, the odd
-// lane h_j of column n + 1, each from one exchanged value; y0, y1 already
-// carry the FP8 scales.
-__device__ __forceinline__ void swiglu_pair(const TcGemm& g, int r, int n, int B, float y0, float y1) {
-  const bool odd = r & 1;
-  const float got = __shfl_xor_sync(0xffffffffu, odd ? y0 : y1, 1);
-  const float gate = odd ? got : y0, up = odd ? y1 : got;
-  const int col = n + (odd ? 1 : 0);
-  if (col < B && r < g.M) {
-    const float h = silu_tc(gate) * up;
-    if (g.h16)
-      static_cast<__nv_bfloat16*>(g.h16)[(size_t)col * (g.M / 2) + (r >> 1)] = __float2bfloat16_rn(h);
-    else
-      g.h_out[(size_t)col * (g.M / 2) + (r >> 1)] = h;
-  }
-}
-
 // One output element (row r of the weights, batch row n) through the store,
 // residual or logits epilogue; y already carries the FP8 scales.
 template <int EPI>
@@ -74,7 +52,7 @@ __device__ __forceinline__ void epi_store(const TcGemm& g, int r, int n, int B, 
     if (EPI == EPI_STORE) {
       g.y[(size_t)n * g.M + r] = y;
     } else if (EPI == EPI_RESID) {
-      g.y[(size_t)n * g.M + r] = res + y;
+      g.y[(size_t)n * g.M + r] = __fadd_rn(res, y);
     } else {
       if (g.zrows)
         g.zrows[(size_t)n * g.M + r] = y;
@@ -109,7 +87,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   int32_t* n_issued = reinterpret_cast<int32_t*>(fail + 1);     // stages whose TMA loads were issued
   int32_t* n_consumed = n_issued + 1;                          // stages the MMA issuer saw land
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int m0 = blockIdx.x * kTileM;
   const int n0 = blockIdx.y * BN;
   const int kblk = KIND_BF16 ? 64 : 128;             // elements per 128-byte K block
@@ -150,8 +128,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tmem_slot;
-  const bool active = true;
+  const uint32_t tmem = uniform(*tmem_slot);
 
   // weight tiles of the first stages do not depend on the previous kernel:
   // in flight before waiting on it; the operand tiles only after
@@ -176,7 +153,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     pre[i] = (EPI == EPI_RESID && n < B && r_ep < g.M) ? __ldcg(g.y + (size_t)n * g.M + r_ep) : 0.f;
   }
 
-  if (active && threadIdx.x == 0) {
+  if (threadIdx.x == 0) {
     // TMA producer
     int ks = 0;
     for (; ks < ns; ++ks) {
@@ -194,38 +171,40 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
     // the first STAGES weight loads went out before the loop in any case
     *n_issued = max(ks, min(ns, STAGES));
-  } else if (active && threadIdx.x == 32) {
-    // MMA issuer: 4 instructions of 32 bytes of K per 128-byte block
-    const uint32_t id = idesc(KIND_BF16, kTileM, BN);
-    bool ok = true;
-    for (int ks = 0; ks < ns && ok; ++ks) {
-      const int s = ks % STAGES;
-      const uint32_t ph = (uint32_t)(ks / STAGES) & 1u;
-      if (!mbar_wait(full + s, ph)) {
-        atomicOr(fail, 2u);
-        ok = false;
-        break;
-      }
-      *n_consumed = ks + 1;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  } else if (warp == 1) {
+    // MMA issuer (one elected lane): 4 instructions of 32 bytes of K per
+    // 128-byte block
+    const uint64_t da = sdesc_sw128(uniform(smem_u32(sA))), db = sdesc_sw128(uniform(smem_u32(sB)));
+    if (elect_one()) {
+      const uint32_t id = idesc(KIND_BF16, kTileM, BN);
+      for (int ks = 0; ks < ns; ++ks) {
+        const int s = ks % STAGES;
+        const uint32_t ph = (uint32_t)(ks / STAGES) & 1u;
+        if (!mbar_wait(full + s, ph)) {
+          atomicOr(fail, 2u);
+          break;
+        }
+        *n_consumed = ks + 1;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-      for (int kk = 0; kk < KP; ++kk) {
-        const int kb = KP * ks + kk;
-        if (kb >= nk) break;                       // a 3D box's block past K: zeros, not multiplied
-        const uint32_t a0 = smem_u32(sA + s * kStageA + (size_t)kk * kTileM * kKBlockBytes);
-        const uint32_t b0 = smem_u32(sB + s * kStageB + (size_t)kk * BN * kKBlockBytes);
+        for (int kk = 0; kk < KP; ++kk) {
+          const int kb = KP * ks + kk;
+          if (kb >= nk) break;                       // a 3D box's block past K: zeros, not multiplied
+          // descriptor addresses count 16 bytes
+          const uint64_t a = da + (uint64_t)((s * kStageA + (size_t)kk * kTileM * kKBlockBytes) >> 4);
+          const uint64_t b = db + (uint64_t)((s * kStageB + (size_t)kk * BN * kKBlockBytes) >> 4);
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          mma_issue(KIND_BF16, tmem, sdesc_sw128(a0 + 32 * k), sdesc_sw128(b0 + 32 * k), id, (kb | k) ? 1u : 0u);
+          for (int k = 0; k < 4; ++k) mma_issue(KIND_BF16, tmem, a + 2 * k, b + 2 * k, id, (kb | k) ? 1u : 0u);
+        }
+        mma_commit(empty + s);
       }
-      mma_commit(empty + s);
+      mma_commit(done);
     }
-    mma_commit(done);
   }
   __syncwarp();
   // accumulator ready (or the pipeline gave up)
-  bool ready = active;
-  if (active && !mbar_wait(done, 0)) {
+  bool ready = true;
+  if (!mbar_wait(done, 0)) {
     atomicOr(fail, 4u);
     ready = false;
   }
@@ -253,12 +232,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         const int n = n0 + c_ep + c0 + i;
-        if (!KIND_BF16) v[i] *= ws * (n < B ? __ldg(g.x_scale + n) : 0.f);
+        if (!KIND_BF16) v[i] = __fmul_rn(v[i], __fmul_rn(ws, n < B ? __ldg(g.x_scale + n) : 0.f));
         if (EPI != EPI_SWIGLU) epi_store<EPI>(g, r, n, B, v[i], pre[c0 + i]);
       }
       if (EPI == EPI_SWIGLU) {
 #pragma unroll
-        for (int i = 0; i < 16; i += 2) swiglu_pair(g, r, n0 + c_ep + c0 + i, B, v[i], v[i + 1]);
+        for (int i = 0; i < 16; i += 2) swiglu_pair(r < g.M, g.M, g.h_out, g.h16, r, n0 + c_ep + c0 + i, B, v[i], v[i + 1]);
       }
     }
     // the remaining columns: the loads of group c + 16 (row scales,
@@ -287,12 +266,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
       for (int i = 0; i < 16; ++i) {
         const int n = n0 + c + i;
-        if (!KIND_BF16) v[i] *= ws * xc[i];
+        if (!KIND_BF16) v[i] = __fmul_rn(v[i], __fmul_rn(ws, xc[i]));
         if (EPI != EPI_SWIGLU) epi_store<EPI>(g, r, n, B, v[i], rc[i]);
       }
       if (EPI == EPI_SWIGLU) {
 #pragma unroll
-        for (int i = 0; i < 16; i += 2) swiglu_pair(g, r, n0 + c + i, B, v[i], v[i + 1]);
+        for (int i = 0; i < 16; i += 2) swiglu_pair(r < g.M, g.M, g.h_out, g.h16, r, n0 + c + i, B, v[i], v[i + 1]);
       }
     }
   }

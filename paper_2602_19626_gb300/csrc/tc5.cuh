@@ -52,6 +52,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
   return false;
 }
 
+// Fetch a tensor map ahead of its first use.
+__device__ __forceinline__ void prefetch_tmap(const void* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
+
 // 2D tiled TMA load of the box at (c0, c1) into shared memory, completing
 // its bytes on `bar`.
 __device__ __forceinline__ void tma_load_2d(void* dst, const void* map, uint64_t* bar, int c0, int c1) {
@@ -110,6 +115,19 @@ __host__ __device__ constexpr uint32_t idesc(int kind_bf16, int M, int N, int b_
          | ((uint32_t)(b_mn ? 1 : 0) << 16)            // B major-ness
          | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
+
+// One lane of a converged warp.  Products are issued by an elected lane, with
+// descriptors formed from warp-uniform values (uniform_warp, uniform): the
+// operands of tcgen05.mma live in uniform registers, and under a plain
+// `threadIdx.x == 0` each instruction cost 76 cycles of issue whatever its
+// shape; elected, 43 (M 128, N 32) and 29 (M 64, N 32).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 
 __device__ __forceinline__ void mma_issue(int kind_bf16, uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t id,
                                           uint32_t accum) {
