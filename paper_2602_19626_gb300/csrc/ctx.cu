@@ -745,10 +745,9 @@ extern "C" int nc_ctx_create(const nc_config* cfg, const void* weights, size_t n
       dalloc(ctx, &ctx->d_st, B * sizeof(StreamDev)))
     return bail(NC_ENOMEM);
   if (D.kv_bf16) {
-    attn_t5_scratch(D, (int)B, ctx->P, &D.attn_part_cap, &D.attn_tickets);
-    if (dalloc(ctx, &D.attn_part, D.attn_part_cap * 4) || dalloc(ctx, &D.attn_ticket, (size_t)D.attn_tickets * 4))
-      return bail(NC_ENOMEM);
-    if (cudaMemset(D.attn_ticket, 0, (size_t)D.attn_tickets * 4) != cudaSuccess) return bail(NC_ECUDA);
+    D.attn_part_cap = attn_t5_scratch(D, ctx->P);
+    if (ctx->P > 0 && dalloc(ctx, &D.attn_part, D.attn_part_cap * 4)) return bail(NC_ENOMEM);
+    if (prepare_attn_dec() != cudaSuccess) return bail(NC_ECUDA);
     if (ctx->P > 0 && dalloc(ctx, &D.q16, (size_t)ctx->P * D.hq * kHeadDim * 2)) return bail(NC_ENOMEM);
     // the attention loads 64-row boxes of the KV rings through one TMA map per slot
     void* maps = nullptr;
@@ -1230,6 +1229,7 @@ static int step_common(nc_ctx* ctx, int n, const int32_t* ids, const int32_t* pr
   const bool dev_out = cdf_out && is_device_ptr(cdf_out);
   Batch b = make_batch(ctx);
   b.obs = nullptr;
+  for (int k : si) b.len_max = std::max(b.len_max, ctx->slots[k].max_len);
   NC_TRY(launch_model(ctx, b));
   VocabIO io{};
   io.cdf = dev_out ? cdf_out : ctx->cdf;
@@ -1664,6 +1664,7 @@ static int encode_device(nc_ctx* ctx, int n, const std::vector<int>& slot_of, co
   if (m >= 2) return encode_prefill(ctx, n, m, tok_dev, offs_dev, lens_dev, lens_h, intervals, stride, trace, probe);
   Batch b = make_batch(ctx);
   b.Bmax = n;
+  b.len_max = max_len;
   VocabIO io = probe;
   io.predict = 1;
   io.update = 1;
@@ -2071,6 +2072,7 @@ extern "C" int nc_decode(nc_ctx* ctx, const uint8_t* in, size_t nbytes, int32_t*
   int64_t max_len = recs[order[0]].ntok;
   Batch b = make_batch(ctx);
   b.Bmax = n;
+  b.len_max = max_len;
   do {
     if (cudaMemcpyAsync(ctx->d_slots, ctx->h_i32 + 1, (size_t)n * 4, cudaMemcpyHostToDevice, s) != cudaSuccess) {
       st = fail_cuda(ctx, cudaErrorUnknown, "slot upload");

@@ -94,15 +94,13 @@ struct Dims {
   int log2T;
   uint32_t floor;
   float alpha, eta;
-  // tensor-core attention over a BF16 cache: per (tile, KV head) the chunks'
-  // partial results and the ticket that picks the CTA merging them
+  // tensor-core prefill attention over a BF16 cache: per (tile, KV head) the
+  // chunks' partial results
   const void* kv_tmap;      // [max_streams] TMA maps (kTmapBytes each) of the slots' BF16 KV
                             // rings as 64-wide rows; nullptr: the attention copies rows itself
   void* q16;                // [prefill_rows][hq * 64] BF16 rotated 1/8-scaled queries of a prefill
   float* attn_part;         // attn_part_cap floats
-  int32_t* attn_ticket;     // attn_tickets counters, zero between launches
   size_t attn_part_cap;
-  int attn_tickets;
 };
 
 // Weights of one dense projection in the storage format.
@@ -138,6 +136,9 @@ struct Batch {
   // wait on the previous kernel.
   const float* z_in;
   const int32_t* z_idx;
+  // Decode rows: a bound of the lengths of their streams (0: none known).
+  // The attention's cluster holds the chunks of the longest window.
+  int64_t len_max;
 };
 
 // (cos, sin) of position a for rotation pair dd from the RoPE table: the
@@ -282,11 +283,14 @@ cudaError_t launch_prepare_prefill(const Batch& b, int n_streams, int m, int V, 
 // k, v appended by the kernel) or prefill rows (b.pm consecutive positions
 // per stream, appended before), into attn_out or, when out16 is set, BF16
 // into out16.  A row's result does not depend on the other rows.
-// D.attn_part / D.attn_ticket must hold what attn_t5_scratch gives for the
-// context's largest batches (tickets zeroed once).
+// A prefill needs D.attn_part (attn_t5_scratch floats) and D.q16.
 cudaError_t launch_attn_t5(const Dims& D, const Batch& b, int layer, const float* qkv, float* attn_out, void* out16,
                            cudaStream_t s);
-void attn_t5_scratch(const Dims& D, int max_streams, int prefill_rows, size_t* part_floats, int* tickets);
+size_t attn_t5_scratch(const Dims& D, int prefill_rows);
+// Its decode rows (k_attn_dec.cu).
+cudaError_t launch_attn_dec(const Dims& D, const Batch& b, int layer, const float* qkv, float* attn_out, void* out16,
+                            cudaStream_t s);
+cudaError_t prepare_attn_dec();
 // Prefill with a BF16 cache: rotate and append every row's k, v to the ring
 // of `layer` and write its rotated, 1/8-scaled BF16 queries to D.q16.
 cudaError_t launch_kv_append_t5(const Dims& D, const Batch& b, int layer, const float* qkv, cudaStream_t s);
