@@ -155,6 +155,71 @@ __device__ void prologue(const Dims& D, Src src, const float* gain, int cols, in
   sync();
 }
 
+// The prologue of rows of at most NT XV columns by a block of NT = 128
+// threads, each row's values held in registers between the sum of squares
+// and the copy to shared memory; the same sums in the same order (value i of
+// thread t is column t + 128 i: even i belong to virtual thread t, odd i to
+// t + 128).  gv: the thread's gains.
+template <bool RMS, int BT, int XV, int NT, typename Src>
+__device__ __forceinline__ void prologue_held(const Dims& D, Src src, const float (&gv)[XV ? XV : 1], int cols, int b0,
+                                              int nb, float* xs, ProScratch& ps, int tid) {
+  static_assert(NT == kRed / 2, "two virtual threads per thread");
+  float x[BT][XV ? XV : 1];
+#pragma unroll
+  for (int bt = 0; bt < BT; ++bt)
+    if (bt < nb) {
+#pragma unroll
+      for (int i = 0; i < XV; ++i) x[bt][i] = tid + NT * i < cols ? src(b0 + bt, tid + NT * i) : 0.f;
+    }
+  if (RMS) {
+#pragma unroll
+    for (int bt = 0; bt < BT; ++bt) {
+      if (bt < nb) {
+        float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+        for (int i = 0; i < XV; ++i) {               // zeros past the row add nothing
+          if (i & 1) s1 = fmaf(x[bt][i], x[bt][i], s1);
+          else s0 = fmaf(x[bt][i], x[bt][i], s0);
+        }
+        s0 = warp_sum(s0);
+        s1 = warp_sum(s1);
+        if ((tid & 31) == 0) {
+          ps.red[tid >> 5][bt] = s0;
+          ps.red[(tid >> 5) + NT / 32][bt] = s1;
+        }
+      }
+    }
+    __syncthreads();
+    if (BT > 1) {
+      if (tid < nb) {
+        float ss = 0.f;
+        for (int w = 0; w < kRed / 32; ++w) ss += ps.red[w][tid];
+        ps.inv[tid] = 1.0f / sqrtf(ss / (float)cols + D.eps);
+      }
+      __syncthreads();
+    }
+  }
+#pragma unroll
+  for (int bt = 0; bt < BT; ++bt)
+    if (bt < nb) {
+      float inv = 1.f;
+      if (RMS) {
+        if (BT > 1) {
+          inv = ps.inv[bt];
+        } else {                                     // every thread forms it: no second barrier
+          float ss = 0.f;
+#pragma unroll
+          for (int w = 0; w < kRed / 32; ++w) ss += ps.red[w][0];
+          inv = 1.0f / sqrtf(ss / (float)cols + D.eps);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < XV; ++i)
+        if (tid + NT * i < cols) xs[bt * cols + tid + NT * i] = RMS ? x[bt][i] * inv * gv[i] : x[bt][i];
+    }
+  __syncthreads();
+}
+
 // Rows of row pair rp (odd row counts duplicate the last row, which is not
 // written back).
 __device__ __forceinline__ void rowpair_rows(const Mat& m, int rp, int& r0, int& r1, bool& has1) {
@@ -195,11 +260,11 @@ struct GemvOut {
 // One row pair for streams b0 .. b0 + nb - 1: lane l accumulates the weight
 // vectors l, l + 32, ... of both rows in increasing order (the held ones, then
 // the rest of a long row), a fixed xor tree sums the lanes, lane bt writes
-// stream b0 + bt.
+// stream b0 + bt (EPI_RESID: added to its residuals res).
 template <int FMT, int EPI, int HOLD = kHold, int BT = kBT>
 __device__ __forceinline__ void gemv_rowpair(const Mat& m, int rp, const float* xs, int b0, int nb,
                                              const uint4 (&h0)[HOLD], const uint4 (&h1)[HOLD], int lane,
-                                             const GemvOut& out) {
+                                             float2 res, const GemvOut& out) {
   using W = WFmt<FMT>;
   constexpr int VW = W::VW;
   int r0, r1;
@@ -277,11 +342,8 @@ __device__ __forceinline__ void gemv_rowpair(const Mat& m, int rp, const float* 
           if (has1) out.y[(size_t)j * m.rows + r1] = y1;
         } else if (EPI == EPI_RESID) {
           float* p0 = out.y + (size_t)j * m.rows + r0;
-          *p0 = __ldcg(p0) + y0;
-          if (has1) {
-            float* p1 = out.y + (size_t)j * m.rows + r1;
-            *p1 = __ldcg(p1) + y1;
-          }
+          *p0 = res.x + y0;
+          if (has1) p0[1] = res.y + y1;
         } else if (EPI == EPI_SWIGLU) {
           out.y[(size_t)j * (m.rows / 2) + r0 / 2] = silu(y0) * y1;
         } else {
