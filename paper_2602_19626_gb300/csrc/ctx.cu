@@ -119,12 +119,17 @@ struct nc_ctx {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_done = nullptr;
   cudaEvent_t ev_fwd[kCodeSets] = {}, ev_voc[kCodeSets] = {};
   uint32_t* cdf = nullptr;
-  int32_t* d_slots = nullptr;
+  // a step's row count, slots and observed tokens: one block laid out as the
+  // head of h_i32, so that a step takes them in one copy
   int32_t* d_nB = nullptr;
+  int32_t* d_slots = nullptr;
   int32_t* d_obs = nullptr;
-  uint32_t* d_target = nullptr;
-  uint32_t* d_lohi = nullptr;
-  int32_t* d_status = nullptr;       // scratch status for building blocks
+  // a decode step's inputs (row count, coder targets) and outputs (coded
+  // intervals, then tokens), each one copy
+  uint32_t* d_dec_in = nullptr;      // [1 + max_streams]
+  uint32_t* d_dec_out = nullptr;     // [3 max_streams]
+  int32_t* d_status = nullptr;       // [0]: status word of the tensor-core projections
+  int32_t* d_word = nullptr;         // [2]: gathered status of a call's streams, d_status[0]
   int64_t* d_meta = nullptr;         // [3 max_streams] an encoder call's row offsets, lengths, caller rows
   // nc_encode's device tokens and intervals, kept (grown as needed) so that
   // repeated calls reuse the same buffers and the captured pass
@@ -133,9 +138,16 @@ struct nc_ctx {
   uint32_t* enc_iv = nullptr;
   size_t enc_iv_cap = 0;
   // pinned host staging
-  int32_t* h_i32 = nullptr;          // 3 * max_streams + 1
-  uint32_t* h_u32 = nullptr;         // 3 * max_streams: targets, then (lo, hi) pairs
-  int32_t* h_status = nullptr;       // max_streams
+  int32_t* h_i32 = nullptr;          // 1 + 2 max_streams: row count, slots, observed tokens
+  uint32_t* h_u32 = nullptr;         // 1 + 4 max_streams: copies of d_dec_in, then of d_dec_out
+  int32_t* h_status = nullptr;       // [2]: d_word's copy
+  // a step's model forward (nc_step_cdf, nc_step_probe) as a captured graph,
+  // one per cluster size of the decode attention; captured at the second
+  // step that needs it, so that a single step pays for no capture
+  struct StepGraph {
+    int uses = 0;
+    cudaGraphExec_t ge = nullptr;
+  } step_graph[4];
 
   // tensor-core path
   std::vector<TcMat> tc;             // per layer: qkv, o, gate/up, down; then the LM head
@@ -165,7 +177,6 @@ struct nc_ctx {
   cudaGraphExec_t pass_graph = nullptr;
 
   StreamDev* d_st = nullptr;
-  std::vector<StreamDev> h_st;
   std::vector<Slot> slots;
   std::unordered_map<int32_t, int> id2slot;
 };
@@ -359,6 +370,8 @@ extern "C" void nc_ctx_destroy(nc_ctx* ctx) {
   cudaFreeHost(ctx->h_u32);
   cudaFreeHost(ctx->h_status);
   if (ctx->pass_graph) cudaGraphExecDestroy(ctx->pass_graph);
+  for (auto& sg : ctx->step_graph)
+    if (sg.ge) cudaGraphExecDestroy(sg.ge);
   cudaFree(ctx->enc_tok);
   cudaFree(ctx->enc_iv);
   for (cudaEvent_t e : {ctx->ev_fork, ctx->ev_join, ctx->ev_done, ctx->ev_fwd[0], ctx->ev_fwd[1], ctx->ev_fwd[2],
@@ -739,11 +752,12 @@ extern "C" int nc_ctx_create(const nc_config* cfg, const void* weights, size_t n
   if (dalloc(ctx, &ctx->x, RA * D.d * 4) || dalloc(ctx, &ctx->qkv, RA * D.qkv_rows * 4) ||
       dalloc(ctx, &ctx->attn_out, RA * D.hq * kHeadDim * 4) ||
       dalloc(ctx, &ctx->h, RA * D.F * 4) || dalloc(ctx, &ctx->cdf, B * (D.V + 1) * 4) ||
-      dalloc(ctx, &ctx->d_slots, B * 4) || dalloc(ctx, &ctx->d_nB, 16) ||
-      dalloc(ctx, &ctx->d_obs, B * 4) || dalloc(ctx, &ctx->d_target, B * 4) ||
-      dalloc(ctx, &ctx->d_lohi, B * 8) || dalloc(ctx, &ctx->d_status, B * 4) || dalloc(ctx, &ctx->d_meta, B * 24) ||
-      dalloc(ctx, &ctx->d_st, B * sizeof(StreamDev)))
+      dalloc(ctx, &ctx->d_nB, (1 + 2 * B) * 4) || dalloc(ctx, &ctx->d_dec_in, (1 + B) * 4) ||
+      dalloc(ctx, &ctx->d_dec_out, B * 12) || dalloc(ctx, &ctx->d_status, B * 4) || dalloc(ctx, &ctx->d_meta, B * 24) ||
+      dalloc(ctx, &ctx->d_word, 16) || dalloc(ctx, &ctx->d_st, B * sizeof(StreamDev)))
     return bail(NC_ENOMEM);
+  ctx->d_slots = ctx->d_nB + 1;
+  ctx->d_obs = ctx->d_nB + 1 + B;
   if (D.kv_bf16) {
     D.attn_part_cap = attn_t5_scratch(D, ctx->P);
     if (ctx->P > 0 && dalloc(ctx, &D.attn_part, D.attn_part_cap * 4)) return bail(NC_ENOMEM);
@@ -756,11 +770,10 @@ extern "C" int nc_ctx_create(const nc_config* cfg, const void* weights, size_t n
       D.kv_tmap = maps;
     }
   }
-  if (cudaMallocHost(&ctx->h_i32, (3 * B + 4) * 4) != cudaSuccess ||
-      cudaMallocHost(&ctx->h_u32, 3 * B * 4) != cudaSuccess ||
-      cudaMallocHost(&ctx->h_status, B * 4) != cudaSuccess)
+  if (cudaMallocHost(&ctx->h_i32, (2 * B + 4) * 4) != cudaSuccess ||
+      cudaMallocHost(&ctx->h_u32, (4 * B + 4) * 4) != cudaSuccess ||
+      cudaMallocHost(&ctx->h_status, 16) != cudaSuccess)
     return bail(NC_ENOMEM);
-  ctx->h_st.assign(B, StreamDev{});
   ctx->slots.assign(B, Slot{});
   if (cudaMemset(ctx->d_st, 0, B * sizeof(StreamDev)) != cudaSuccess) return bail(NC_ECUDA);
   if (cudaMemset(ctx->d_status, 0, B * 4) != cudaSuccess) return bail(NC_ECUDA);
@@ -792,7 +805,7 @@ static int slot_alloc(nc_ctx* ctx, Slot& s, int64_t max_len) {
     // every ring entry finite from the start: the tensor-core attention
     // multiplies the entries past a row's position by zero probabilities
     const size_t kvb = (size_t)D.n_layers * 2 * D.hkv * D.L * kHeadDim * (D.kv_bf16 ? 2 : 4);
-    NC_TRY(cudaMemset(s.kv, 0, kvb));
+    NC_TRY(cudaMemsetAsync(s.kv, 0, kvb, ctx->stream));
     if (D.kv_tmap) {
       CUtensorMap map;
       if (!tc_encode_tmap(&map, s.kv, 2, kHeadDim, (int64_t)D.n_layers * 2 * D.hkv * D.L, 64))
@@ -839,9 +852,6 @@ static int open_slot(nc_ctx* ctx, int32_t id, int64_t max_len, int* slot_out) {
   if (st != NC_OK) return st;
   const Dims& D = ctx->D;
   cudaStream_t cs = ctx->stream;
-  NC_TRY(cudaMemsetAsync(s.bias, 0, (size_t)D.V * 4, cs));
-  NC_TRY(cudaMemsetAsync(s.uni, 0, (size_t)D.V * 4, cs));
-  for (int k = 0; k < D.order; ++k) NC_TRY(cudaMemsetAsync(s.keys[k], 0xFF, (size_t)s.cap_hash * 8, cs));
   StreamDev sd{};
   sd.n_coded = 0;
   sd.last_tok = 0;   // BOS
@@ -864,9 +874,8 @@ static int open_slot(nc_ctx* ctx, int32_t id, int64_t max_len, int* slot_out) {
   sd.uni = s.uni;
   sd.z = s.z;
   sd.kv = s.kv;
-  ctx->h_st[si] = sd;
-  NC_TRY(cudaMemcpyAsync(ctx->d_st + si, &ctx->h_st[si], sizeof(StreamDev), cudaMemcpyHostToDevice, cs));
-  NC_TRY(cudaStreamSynchronize(cs));
+  // fresh state by one kernel in stream order (no copy, no synchronisation)
+  NC_TRY(launch_open(sd, ctx->d_st + si, D.V, D.order, s.cap_hash, cs));
   s.open = true;
   s.awaiting_update = false;
   s.id = id;
@@ -1155,7 +1164,8 @@ static void step_cost(const nc_ctx* ctx, int B, double ctx_sum, double kv_unique
 
 // Host-side checks and staging of a batch of open streams.
 static int stage_batch(nc_ctx* ctx, int n, const int32_t* ids, std::vector<int>* slot_idx,
-                       bool want_awaiting) {
+                       const int32_t* observed) {
+  const bool want_awaiting = observed != nullptr;
   if (n < 1 || n > ctx->cfg.max_streams || !ids) return fail(ctx, NC_EINVAL, "bad stream count or ids");
   slot_idx->resize(n);
   for (int j = 0; j < n; ++j) {
@@ -1173,34 +1183,29 @@ static int stage_batch(nc_ctx* ctx, int n, const int32_t* ids, std::vector<int>*
     return fail(ctx, NC_EINVAL, "duplicate stream id");
   ctx->h_i32[0] = n;
   for (int j = 0; j < n; ++j) ctx->h_i32[1 + j] = (*slot_idx)[j];
-  NC_TRY(cudaMemcpyAsync(ctx->d_nB, ctx->h_i32, 4, cudaMemcpyHostToDevice, ctx->stream));
-  NC_TRY(cudaMemcpyAsync(ctx->d_slots, ctx->h_i32 + 1, (size_t)n * 4, cudaMemcpyHostToDevice, ctx->stream));
+  // the observed tokens of an update follow the slots (at max_streams)
+  size_t words = 1 + (size_t)n;
+  if (observed) {
+    std::memcpy(ctx->h_i32 + 1 + ctx->cfg.max_streams, observed, (size_t)n * 4);
+    words = 1 + (size_t)ctx->cfg.max_streams + n;
+  }
+  NC_TRY(cudaMemcpyAsync(ctx->d_nB, ctx->h_i32, words * 4, cudaMemcpyHostToDevice, ctx->stream));
   return NC_OK;
 }
 
-// Read and clear the sticky status words of the given slots (and the
-// context-wide word of the tensor-core GEMMs).
+// Read and clear the sticky status words of the n streams in d_slots (and
+// read the context-wide word of the tensor-core GEMMs): one kernel gathers
+// them, one copy brings them.
 static int check_status(nc_ctx* ctx, const std::vector<int>& slot_idx) {
-  const size_t off = offsetof(StreamDev, status);
-  if (ctx->cfg.path == NC_PATH_TC) {
-    int32_t w = 0;
-    NC_TRY(cudaMemcpyAsync(&w, ctx->d_status, 4, cudaMemcpyDeviceToHost, ctx->stream));
-    NC_TRY(cudaStreamSynchronize(ctx->stream));
-    if (w) {
-      ctx->poisoned = true;
-      return fail(ctx, NC_ETIMEOUT, "a tensor-core pipeline wait gave up");
-    }
-  }
-  for (size_t j = 0; j < slot_idx.size(); ++j)
-    NC_TRY(cudaMemcpyAsync(ctx->h_status + j, reinterpret_cast<char*>(ctx->d_st + slot_idx[j]) + off, 4,
-                           cudaMemcpyDeviceToHost, ctx->stream));
+  NC_TRY(launch_gather_status(ctx->d_st, ctx->d_slots, (int)slot_idx.size(), ctx->d_status, ctx->d_word, ctx->stream));
+  NC_TRY(cudaMemcpyAsync(ctx->h_status, ctx->d_word, 8, cudaMemcpyDeviceToHost, ctx->stream));
   NC_TRY(cudaStreamSynchronize(ctx->stream));
-  int32_t any = 0;
-  for (size_t j = 0; j < slot_idx.size(); ++j) any |= ctx->h_status[j];
+  const int32_t any = ctx->h_status[0];
+  if (ctx->cfg.path == NC_PATH_TC && ctx->h_status[1]) {
+    ctx->poisoned = true;
+    return fail(ctx, NC_ETIMEOUT, "a tensor-core pipeline wait gave up");
+  }
   if (any) {
-    for (size_t j = 0; j < slot_idx.size(); ++j)
-      NC_TRY(cudaMemsetAsync(reinterpret_cast<char*>(ctx->d_st + slot_idx[j]) + off, 0, 4, ctx->stream));
-    NC_TRY(cudaStreamSynchronize(ctx->stream));
     if (any & ST_TIMEOUT) {
       ctx->poisoned = true;
       return fail(ctx, NC_ETIMEOUT, "a bounded device wait gave up");
@@ -1212,6 +1217,28 @@ static int check_status(nc_ctx* ctx, const std::vector<int>& slot_idx) {
   return NC_OK;
 }
 
+// The model forward of a step over the staged rows, replayed from a graph.
+static cudaError_t step_model(nc_ctx* ctx, const Batch& b) {
+  nc_ctx::StepGraph& sg = ctx->step_graph[attn_dec_class(ctx->D, b)];
+  if (sg.uses == 0 || (sg.uses > 1 && !sg.ge)) {   // the first step, or no graph could be captured
+    sg.uses = std::max(sg.uses, 1);
+    return launch_model(ctx, b);
+  }
+  if (sg.uses++ == 1) {
+    cudaGraph_t g = nullptr;
+    if (cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+      const cudaError_t e = launch_model(ctx, b);
+      const cudaError_t e2 = cudaStreamEndCapture(ctx->stream, &g);
+      if (e != cudaSuccess || e2 != cudaSuccess || cudaGraphInstantiate(&sg.ge, g, 0) != cudaSuccess) sg.ge = nullptr;
+      if (g) cudaGraphDestroy(g);
+    }
+    cudaGetLastError();
+    if (!sg.ge) return launch_model(ctx, b);
+  }
+  sg.uses = 2;
+  return cudaGraphLaunch(sg.ge, ctx->stream);
+}
+
 static int step_common(nc_ctx* ctx, int n, const int32_t* ids, const int32_t* prev, float* z,
                        float* pt, float* png, float* p, uint32_t* cdf_out) {
   if (!ctx) return NC_EINVAL;
@@ -1219,7 +1246,7 @@ static int step_common(nc_ctx* ctx, int n, const int32_t* ids, const int32_t* pr
   if (ctx->poisoned) return fail(ctx, NC_ESTATE, "context poisoned by an earlier CUDA error");
   cudaSetDevice(ctx->cfg.device);
   std::vector<int> si;
-  int st = stage_batch(ctx, n, ids, &si, false);
+  int st = stage_batch(ctx, n, ids, &si, nullptr);
   if (st != NC_OK) return st;
   if (prev) {
     for (int j = 0; j < n; ++j)
@@ -1230,7 +1257,7 @@ static int step_common(nc_ctx* ctx, int n, const int32_t* ids, const int32_t* pr
   Batch b = make_batch(ctx);
   b.obs = nullptr;
   for (int k : si) b.len_max = std::max(b.len_max, ctx->slots[k].max_len);
-  NC_TRY(launch_model(ctx, b));
+  NC_TRY(step_model(ctx, b));
   VocabIO io{};
   io.cdf = dev_out ? cdf_out : ctx->cdf;
   io.probe_z = z;
@@ -1268,11 +1295,8 @@ extern "C" int nc_update_bias(nc_ctx* ctx, int n, const int32_t* stream_ids, con
   for (int j = 0; j < n; ++j)
     if (observed[j] < 0 || observed[j] >= ctx->D.V) return fail(ctx, NC_EINVAL, "observed token out of range");
   std::vector<int> si;
-  int st = stage_batch(ctx, n, stream_ids, &si, true);
+  int st = stage_batch(ctx, n, stream_ids, &si, observed);
   if (st != NC_OK) return st;
-  std::memcpy(ctx->h_i32 + 1 + ctx->cfg.max_streams, observed, (size_t)n * 4);
-  NC_TRY(cudaMemcpyAsync(ctx->d_obs, ctx->h_i32 + 1 + ctx->cfg.max_streams, (size_t)n * 4,
-                         cudaMemcpyHostToDevice, ctx->stream));
   Batch b = make_batch(ctx);
   VocabIO io{};
   io.update = 1;
@@ -2083,22 +2107,24 @@ extern "C" int nc_decode(nc_ctx* ctx, const uint8_t* in, size_t nbytes, int32_t*
     // memory, the model, the CDFs, the search, the updates, the coded
     // intervals and tokens out.  Captured once in a CUDA graph and replayed
     // per position; the copies read and write the same pinned buffers.
+    uint32_t* h_in = ctx->h_u32;
+    uint32_t* h_out = ctx->h_u32 + 1 + ctx->cfg.max_streams;
+    int32_t* obs = reinterpret_cast<int32_t*>(ctx->d_dec_out + 2 * n);
+    b.nB = reinterpret_cast<const int32_t*>(ctx->d_dec_in);
+    b.obs = obs;
     auto one_step = [&]() -> cudaError_t {
-      cudaError_t e = cudaMemcpyAsync(ctx->d_nB, ctx->h_i32, 4, cudaMemcpyHostToDevice, s);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->d_target, ctx->h_u32, (size_t)n * 4, cudaMemcpyHostToDevice, s);
+      cudaError_t e = cudaMemcpyAsync(ctx->d_dec_in, h_in, (1 + (size_t)n) * 4, cudaMemcpyHostToDevice, s);
       if (e == cudaSuccess) e = launch_model(ctx, b);
       VocabIO io{};
       io.cdf = ctx->cdf;
       io.predict = 1;
       if (e == cudaSuccess) e = launch_vocab(D, b, io, s);
-      if (e == cudaSuccess) e = launch_search(b, D.V, ctx->cdf, ctx->d_target, ctx->d_obs, ctx->d_lohi, s);
+      if (e == cudaSuccess) e = launch_search(b, D.V, ctx->cdf, ctx->d_dec_in + 1, obs, ctx->d_dec_out, D.pdl, s);
       VocabIO up{};
       up.update = 1;
       up.ngram = 1;
       if (e == cudaSuccess) e = launch_vocab(D, b, up, s);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->h_u32 + n, ctx->d_lohi, (size_t)n * 8, cudaMemcpyDeviceToHost, s);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->h_i32 + 1 + 2 * ctx->cfg.max_streams, ctx->d_obs, (size_t)n * 4,
-                                                cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(h_out, ctx->d_dec_out, (size_t)n * 12, cudaMemcpyDeviceToHost, s);
       return e;
     };
     cudaGraphExec_t ge = nullptr;
@@ -2115,8 +2141,8 @@ extern "C" int nc_decode(nc_ctx* ctx, const uint8_t* in, size_t nbytes, int32_t*
     int active = n;
     for (int64_t k = 0; k < max_len && st == NC_OK; ++k) {
       while (active > 0 && recs[order[active - 1]].ntok <= k) --active;
-      ctx->h_i32[0] = active;
-      for (int r = 0; r < active; ++r) ctx->h_u32[r] = rans ? rdec[r].target() : dec[r].target();
+      h_in[0] = (uint32_t)active;
+      for (int r = 0; r < active; ++r) h_in[1 + r] = rans ? rdec[r].target() : dec[r].target();
       cudaError_t e = ge ? cudaGraphLaunch(ge, s) : one_step();
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) {
@@ -2124,12 +2150,12 @@ extern "C" int nc_decode(nc_ctx* ctx, const uint8_t* in, size_t nbytes, int32_t*
         break;
       }
       for (int r = 0; r < active; ++r) {
-        const uint32_t lo = ctx->h_u32[n + 2 * r], hi = ctx->h_u32[n + 2 * r + 1];
+        const uint32_t lo = h_out[2 * r], hi = h_out[2 * r + 1];
         if (rans)
           rdec[r].consume(lo, hi);
         else
           dec[r].consume(lo, hi);
-        tokens_out[order[r]][k] = ctx->h_i32[1 + 2 * ctx->cfg.max_streams + r];
+        tokens_out[order[r]][k] = (int32_t)h_out[2 * n + r];
       }
     }
     if (ge) cudaGraphExecDestroy(ge);

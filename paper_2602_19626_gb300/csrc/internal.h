@@ -291,6 +291,14 @@ size_t attn_t5_scratch(const Dims& D, int prefill_rows);
 cudaError_t launch_attn_dec(const Dims& D, const Batch& b, int layer, const float* qkv, float* attn_out, void* out16,
                             cudaStream_t s);
 cudaError_t prepare_attn_dec();
+// log2 of its cluster size for the launch's rows (Batch::len_max).
+int attn_dec_class(const Dims& D, const Batch& b);
+// Fresh state of a stream: bias, unigram counts and the hash index cleared,
+// *dst = sd (Algorithm 1, "init").
+cudaError_t launch_open(const StreamDev& sd, StreamDev* dst, int V, int order, int64_t cap_hash, cudaStream_t s);
+// out[0] = the OR of the status words of st[slots[0 .. n - 1]], cleared; out[1] = *tc_status.
+cudaError_t launch_gather_status(StreamDev* st, const int32_t* slots, int n, const int32_t* tc_status, int32_t* out,
+                                 cudaStream_t s);
 // Prefill with a BF16 cache: rotate and append every row's k, v to the ring
 // of `layer` and write its rotated, 1/8-scaled BF16 queries to D.q16.
 cudaError_t launch_kv_append_t5(const Dims& D, const Batch& b, int layer, const float* qkv, cudaStream_t s);
@@ -299,7 +307,7 @@ cudaError_t launch_kv_append(const Dims& D, const Batch& b, int layer, const flo
 // Decoder: row j's symbol is the s with cdf[s] <= target[j] < cdf[s+1]; writes
 // obs[j] = s and lohi[2j..2j+1] = (cdf[s], cdf[s+1]).
 cudaError_t launch_search(const Batch& b, int V, const uint32_t* cdf, const uint32_t* target,
-                          int32_t* obs, uint32_t* lohi, cudaStream_t s);
+                          int32_t* obs, uint32_t* lohi, bool pdl, cudaStream_t s);
 cudaError_t launch_convert_weights(const float* src, void* dst, float* scale, int64_t rows,
                                    int64_t cols, int fmt, cudaStream_t s);
 cudaError_t launch_interleave_f32(const float* gate, const float* up, float* dst, int64_t rows,

@@ -321,16 +321,22 @@ cudaError_t prepare_attn_dec() {
   return e;
 }
 
-cudaError_t launch_attn_dec(const Dims& D, const Batch& b, int layer, const float* qkv, float* attn_out, void* out16,
-                            cudaStream_t s) {
-  const AttnIO io{qkv, attn_out, out16};
+int attn_dec_class(const Dims& D, const Batch& b) {
   // chunks of the longest window a row of this launch may reach
   const int64_t len = b.len_max > 0 && b.len_max < D.L ? b.len_max : D.L;
   const int nch = (int)((len + kT5Chunk - 1) / kT5Chunk);
-  if (nch <= 1) return launch_dec_s<1>(D, b, layer, io, s);
-  if (nch <= 2) return launch_dec_s<2>(D, b, layer, io, s);
-  if (nch <= 4) return launch_dec_s<4>(D, b, layer, io, s);
-  return launch_dec_s<8>(D, b, layer, io, s);
+  return nch <= 1 ? 0 : nch <= 2 ? 1 : nch <= 4 ? 2 : 3;
+}
+
+cudaError_t launch_attn_dec(const Dims& D, const Batch& b, int layer, const float* qkv, float* attn_out, void* out16,
+                            cudaStream_t s) {
+  const AttnIO io{qkv, attn_out, out16};
+  switch (attn_dec_class(D, b)) {
+    case 0: return launch_dec_s<1>(D, b, layer, io, s);
+    case 1: return launch_dec_s<2>(D, b, layer, io, s);
+    case 2: return launch_dec_s<4>(D, b, layer, io, s);
+    default: return launch_dec_s<8>(D, b, layer, io, s);
+  }
 }
 
 }  // namespace nc

@@ -1811,27 +1811,58 @@ __global__ void __launch_bounds__(kVocabThreads)
   }
 }
 
-// One warp per row: binary search of the decoder's target count in the CDF.
+// Fresh state of one stream (grid-stride): the bias and unigram counts zero,
+// the hash index of every order empty, the stream's record by value.
+__global__ void k_open(StreamDev sd, StreamDev* dst, int V, int order, int64_t cap) {
+  const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, n = gridDim.x * (int64_t)blockDim.x;
+  for (int64_t i = i0; i < V; i += n) {
+    sd.bias[i] = 0.f;
+    sd.uni[i] = 0;
+  }
+  for (int k = 0; k < order; ++k)
+    for (int64_t i = i0; i < cap; i += n) sd.keys[k][i] = kEmptyKey;
+  if (i0 == 0) *dst = sd;
+}
+
+__global__ void k_gather_status(StreamDev* st, const int32_t* slots, int n, const int32_t* tc_status, int32_t* out) {
+  int32_t w = 0;
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    int32_t* p = &st[slots[j]].status;
+    const int32_t v = *p;
+    if (v) *p = 0;
+    w |= v;
+  }
+  const int any_n = __syncthreads_or(w & ST_NUMERIC), any_f = __syncthreads_or(w & ST_TABLE_FULL),
+            any_b = __syncthreads_or(w & ST_BAD_TOKEN), any_t = __syncthreads_or(w & ST_TIMEOUT);
+  if (threadIdx.x == 0) {
+    out[0] = (any_n ? ST_NUMERIC : 0) | (any_f ? ST_TABLE_FULL : 0) | (any_b ? ST_BAD_TOKEN : 0) | (any_t ? ST_TIMEOUT : 0);
+    out[1] = *tc_status;
+  }
+}
+
+// One warp per row: search of the decoder's target count in the CDF, 32
+// probes a round (49,152 symbols: 4 dependent loads instead of the 16 of a
+// binary search, 8.0 us a launch with those).
 __global__ void k_search(Batch b, int V, const uint32_t* cdf, const uint32_t* target, int32_t* obs,
                          uint32_t* lohi) {
-  pdl_wait();
-  pdl_trigger();
   const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (j >= *b.nB || lane != 0) return;
+  pdl_wait();
+  pdl_trigger();
+  if (j >= *b.nB) return;
   const uint32_t* row = cdf + (size_t)j * (V + 1);
   const uint32_t t = target[j];
-  int lo = 0, hi = V - 1;                // largest s with row[s] <= t
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (row[mid] <= t)
-      lo = mid;
-    else
-      hi = mid - 1;
+  int lo = 0, n = V;                     // the largest s with row[s] <= t is in [lo, lo + n); row[0] = 0
+  while (n > 1) {
+    const int step = (n + 31) / 32, at = lane * step;
+    const bool le = at < n && row[lo + at] <= t;
+    const unsigned m = __ballot_sync(0xffffffffu, le);
+    const int last = m ? 31 - __clz(m) : 0;          // the CDF does not decrease
+    lo += last * step;
+    n = min(step, n - last * step);
   }
-  obs[j] = lo;
-  lohi[2 * j] = row[lo];
-  lohi[2 * j + 1] = row[lo + 1];
+  if (lane < 2) lohi[2 * j + lane] = row[lo + lane];
+  if (lane == 0) obs[j] = lo;
 }
 
 }  // namespace
@@ -2028,12 +2059,23 @@ cudaError_t launch_floor_counts(const float* p, int64_t n, uint32_t K, uint32_t 
   return cudaGetLastError();
 }
 
+cudaError_t launch_open(const StreamDev& sd, StreamDev* dst, int V, int order, int64_t cap_hash, cudaStream_t s) {
+  const int64_t most = order > 0 ? std::max<int64_t>(V, cap_hash) : V;
+  k_open<<<(unsigned)std::min<int64_t>((most + 255) / 256, 608), 256, 0, s>>>(sd, dst, V, order, cap_hash);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gather_status(StreamDev* st, const int32_t* slots, int n, const int32_t* tc_status, int32_t* out,
+                                 cudaStream_t s) {
+  k_gather_status<<<1, std::min(1024, (n + 31) / 32 * 32), 0, s>>>(st, slots, n, tc_status, out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_search(const Batch& b, int V, const uint32_t* cdf, const uint32_t* target,
-                          int32_t* obs, uint32_t* lohi, cudaStream_t s) {
+                          int32_t* obs, uint32_t* lohi, bool pdl, cudaStream_t s) {
   const int threads = 128;
   const int blocks = (b.Bmax * 32 + threads - 1) / threads;
-  k_search<<<blocks, threads, 0, s>>>(b, V, cdf, target, obs, lohi);
-  return cudaGetLastError();
+  return launch_kernel(k_search, dim3(blocks), dim3(threads), 0, s, pdl, b, V, cdf, target, obs, lohi);
 }
 
 cudaError_t launch_mix_nll(const float* z, const float* b, const float* png, const float* theta,
