@@ -11,6 +11,7 @@
 #include <string>
 #include <thread>
 #include <map>
+#include <mutex>
 #include <unordered_map>
 #include <vector>
 
@@ -2222,26 +2223,89 @@ extern "C" int nc_launch_chain_floor(int device, int n_links, int blocks, int th
   return e == cudaSuccess ? NC_OK : NC_ECUDA;
 }
 
+// Status words of the building blocks that return one to the host: a fixed
+// array of the library image (1 KB per device that loads it), a word leased
+// for the length of a call, so that calls on several threads, streams and
+// devices each have their own and none allocates (a cudaMalloc and cudaFree
+// cost more than the kernels).  A word is zero when it is leased; a call that
+// raised it clears it, and one that failed to read it keeps it out of use.
+// With every word leased a call allocates its own.
+static __device__ int32_t g_words[256];
+namespace {
+constexpr int kWords = 256, kWordDevices = 64;
+std::mutex g_words_mu;
+std::vector<int> g_words_free[kWordDevices];
+bool g_words_init[kWordDevices] = {};
+
+struct WordLease {
+  int dev = -1, slot = -1;
+  int32_t* p = nullptr;
+  bool owned = false;                              // allocated by this call
+  cudaError_t take() {
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < kWordDevices) {
+      std::lock_guard<std::mutex> lock(g_words_mu);
+      auto& f = g_words_free[dev];
+      if (!g_words_init[dev]) {
+        for (int i = 0; i < kWords; ++i) f.push_back(i);
+        g_words_init[dev] = true;
+      }
+      if (!f.empty()) {
+        slot = f.back();
+        f.pop_back();
+      }
+    }
+    void* q = nullptr;
+    if (slot >= 0) {
+      e = cudaGetSymbolAddress(&q, g_words);
+      if (e == cudaSuccess) p = static_cast<int32_t*>(q) + slot;
+      else give();
+      return e;
+    }
+    owned = true;
+    e = dev_malloc(&p, 4);
+    return e == cudaSuccess ? cudaMemset(p, 0, 4) : e;
+  }
+  // Read the word after the work on s, clear it if raised, give it back.
+  cudaError_t finish(cudaStream_t s, int32_t* out) {
+    *out = 0;
+    cudaError_t e = cudaMemcpyAsync(out, p, 4, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && *out && !owned) {
+      e = cudaMemsetAsync(p, 0, 4, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    }
+    if (e == cudaSuccess || owned) give();
+    return e;
+  }
+  void give() {
+    if (owned) {
+      cudaFree(p);
+    } else if (slot >= 0) {
+      std::lock_guard<std::mutex> lock(g_words_mu);
+      g_words_free[dev].push_back(slot);
+    }
+    slot = -1;
+    owned = false;
+  }
+};
+}  // namespace
+
 extern "C" int nc_probs_to_cdf(const float* p, int n, int V, int log2_total, uint32_t floor_c, uint32_t* cdf,
                                void* stream) {
   if (!p || !cdf || n < 1 || V < 2 || V > 65535 || log2_total < 1 || log2_total > 24 || floor_c < 1 ||
       (uint64_t)V * floor_c >= (1ull << log2_total))
     return NC_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  int32_t* status = nullptr;
-  if (dev_malloc(&status, (size_t)n * 4) != cudaSuccess) return NC_ENOMEM;
-  int rc = NC_OK;
-  std::vector<int32_t> hs(n);
-  if (cudaMemsetAsync(status, 0, (size_t)n * 4, s) != cudaSuccess ||
-      launch_probs_to_cdf(p, n, V, log2_total, floor_c, cdf, status, s) != cudaSuccess ||
-      cudaMemcpyAsync(hs.data(), status, (size_t)n * 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
-    rc = NC_ECUDA;
-  cudaFree(status);
-  if (rc == NC_OK)
-    for (int j = 0; j < n; ++j)
-      if (hs[j]) rc = NC_ENUMERIC;
-  return rc;
+  WordLease w;
+  const cudaError_t e = w.take();
+  if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? NC_ENOMEM : NC_ECUDA;
+  const cudaError_t el = launch_probs_to_cdf(p, n, V, log2_total, floor_c, cdf, w.p, false, s);
+  int32_t bad = 0;
+  const cudaError_t ef = w.finish(s, &bad);
+  if (el != cudaSuccess || ef != cudaSuccess) return NC_ECUDA;
+  return bad ? NC_ENUMERIC : NC_OK;
 }
 
 extern "C" int nc_floor_counts(const float* p, int64_t n, uint32_t K, uint32_t floor_c, uint32_t* c, void* stream) {
@@ -2263,11 +2327,9 @@ extern "C" int nc_gemm_tc(const void* W, const void* X, const float* w_scale, co
   t.K = K;
   if (!tc_encode_weights(t, W, esz) || !tc_encode_operand(t, &t.b[0][0], X, esz, N, bn)) return NC_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  int32_t* dev = nullptr;
-  if (dev_malloc(&dev, 8) != cudaSuccess) return NC_ENOMEM;
-  const int32_t h[2] = {N, 0};
-  int rc = NC_OK;
-  int32_t back[2] = {0, 0};
+  WordLease w;
+  const cudaError_t e = w.take();
+  if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? NC_ENOMEM : NC_ECUDA;
   TcGemm g{};
   g.tmap_a = &t.a;
   g.tmap_b = &t.b[0][0];
@@ -2277,18 +2339,15 @@ extern "C" int nc_gemm_tc(const void* W, const void* X, const float* w_scale, co
   g.bn = bn;
   g.kp = t.kp;
   g.kind_bf16 = !fp8;
-  g.nB = dev;
   g.w_scale = w_scale;
   g.x_scale = x_scale;
   g.y = Y;
-  g.status = dev + 1;
-  if (cudaMemcpyAsync(dev, h, 8, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-      launch_gemm_tc(g, EPI_STORE, s, false) != cudaSuccess ||
-      cudaMemcpyAsync(back, dev, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
-    rc = NC_ECUDA;
-  cudaFree(dev);
-  if (rc == NC_OK && back[1]) rc = NC_ETIMEOUT;
-  return rc;
+  g.status = w.p;
+  const cudaError_t el = launch_gemm_tc(g, EPI_STORE, s, false);
+  int32_t gave_up = 0;
+  const cudaError_t ef = w.finish(s, &gave_up);
+  if (el != cudaSuccess || ef != cudaSuccess) return NC_ECUDA;
+  return gave_up ? NC_ETIMEOUT : NC_OK;
 }
 
 extern "C" int nc_ac_encode(const uint32_t* lo, const uint32_t* hi, int64_t n, int log2_total, uint8_t* out,

@@ -12,8 +12,6 @@ constexpr int kHeadDim = 64;           // d_head of the supported models (Sec. 3
 constexpr int kMaxSlots = 64;          // continuation slots per N-gram context (Sec. 3.4)
 constexpr int kMaxOrder = 3;           // N-gram context lengths 1..3
 constexpr int kMaxGroup = 4;           // query heads per KV head supported
-constexpr int kVocabCluster = 8;       // CTAs per row in the standalone quantiser kernels
-constexpr int kVocabThreads = 512;
 constexpr float kSkipBits = 1.5f;      // the skip threshold on the N-gram entropy (Sec. 3.7)
 constexpr unsigned long long kEmptyKey = ~0ull;
 
@@ -321,7 +319,7 @@ struct TcGemm {
   int M, K, Bmax, bn, kind_bf16;
   int kp;                   // 2: both maps 3D ([K blocks][rows][128 B], tc_encode_tmap3), two K blocks
                             // per stage (BF16, K a multiple of 64); otherwise 2D maps, one per stage
-  const int32_t* nB;
+  const int32_t* nB;        // active rows (device scalar), or nullptr: Bmax
   const float* w_scale;     // FP8: [M]
   const float* x_scale;     // FP8: [Bmax]
   float* y;                 // EPI_STORE / EPI_RESID: [Bmax][M]
@@ -375,8 +373,9 @@ cudaError_t prepare_model_kernels(const Dims& D, int fmt);
 cudaError_t prepare_vocab_kernels(const Dims& D);
 cudaError_t prepare_tc_kernels();
 
+// status: a word per row (per_row), or one word that any bad row raises.
 cudaError_t launch_probs_to_cdf(const float* p, int n, int V, int log2T, uint32_t floor,
-                                uint32_t* cdf, int32_t* status, cudaStream_t s);
+                                uint32_t* cdf, int32_t* status, bool per_row, cudaStream_t s);
 cudaError_t launch_floor_counts(const float* p, int64_t n, uint32_t K, uint32_t floor,
                                 uint32_t* c, cudaStream_t s);
 cudaError_t launch_mix_nll(const float* z, const float* b, const float* png, const float* theta,

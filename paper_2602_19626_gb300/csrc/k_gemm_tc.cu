@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
   // the row count was written by the step's prepare kernel, several launches
   // back, so it may be read before the wait on the previous kernel
-  const int B = *g.nB;
+  const int B = g.nB ? *g.nB : g.Bmax;
   if (n0 >= B) return;                            // uniform across the CTA
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {

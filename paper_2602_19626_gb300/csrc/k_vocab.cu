@@ -23,8 +23,6 @@ namespace nc {
 
 namespace {
 
-constexpr int kWarps = kVocabThreads / 32;
-
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -63,56 +61,6 @@ __device__ __forceinline__ uint32_t floor_count(float p, uint32_t K, float Kf, b
   uint32_t q = __float2uint_rz(x);
   if (x >= 16777216.f) q = floor_prod(p, K, bad);
   return q;
-}
-
-struct ArgMax {
-  float v;
-  int i;
-};
-__device__ __forceinline__ ArgMax better(ArgMax a, ArgMax b) {
-  // larger value wins; equal values: lower index wins (first maximum)
-  if (b.v > a.v || (b.v == a.v && b.i < a.i)) return b;
-  return a;
-}
-
-// Shared scratch of one CTA of the standalone kernels: block-reduction
-// slots and the values it publishes to the other CTAs of its cluster.
-template <int NW>
-struct VocabSharedT {
-  static constexpr int kNW = NW;
-  float wm[NW], wsum[NW];
-  unsigned long long wc[NW];
-  ArgMax wa[NW];
-  uint32_t wscan[NW];
-  // published to the cluster
-  unsigned long long cl_csum;
-  ArgMax cl_arg;
-  uint32_t cl_bad;
-  uint32_t cl_total;
-};
-using VocabShared = VocabSharedT<kWarps>;
-
-template <typename Sh>
-__device__ float block_max(float v, Sh& sh) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  v = warp_max(v);
-  if (lane == 0) sh.wm[w] = v;
-  __syncthreads();
-  float r = sh.wm[0];
-  for (int i = 1; i < Sh::kNW; ++i) r = fmaxf(r, sh.wm[i]);
-  __syncthreads();
-  return r;
-}
-template <typename Sh>
-__device__ float block_sum(float v, Sh& sh) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  v = warp_sum(v);
-  if (lane == 0) sh.wsum[w] = v;
-  __syncthreads();
-  float r = 0.f;
-  for (int i = 0; i < Sh::kNW; ++i) r += sh.wsum[i];
-  __syncthreads();
-  return r;
 }
 
 template <int E>
@@ -173,124 +121,6 @@ __device__ __forceinline__ void store_counts(int32_t* dst, int v0, int V, const 
     for (int i = 0; i < E; ++i)
       if (v0 + i < V) dst[v0 + i] = in[i];
   }
-}
-
-// ------------------------------------------------ standalone quantiser rounds
-struct QuantResult {
-  long long resid;          // T - sum of floored counts, added to the first maximum
-  int argmax;
-  bool bad;                 // non-finite / out-of-range probability, or floor underflow
-};
-
-// Floor-quantise the thread's E probabilities into c[], reduce the count sum
-// and the first argmax over the cluster (thread -> warp -> CTA -> ranks in
-// order), and add the residual to the first maximum.
-template <int E, int CL, typename Sh>
-__device__ QuantResult quantise_round(const float (&p)[E], int v0, int V, int log2T, uint32_t floor_c,
-                                      uint32_t (&c)[E], cg::cluster_group& cl, Sh& sh) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const uint32_t T = 1u << log2T;
-  const uint32_t K = T - (uint32_t)V * floor_c;
-  bool bad = false;
-  unsigned long long csum = 0;
-  ArgMax am{-INFINITY, 0x7fffffff};
-#pragma unroll
-  for (int i = 0; i < E; ++i) {
-    const int v = v0 + i;
-    c[i] = 0;
-    if (v < V) {
-      const uint32_t q = floor_count(p[i], K, (float)K, bad);
-      c[i] = q > floor_c ? q : floor_c;
-      csum += c[i];
-      if (p[i] > am.v) am = ArgMax{p[i], v};   // strict: keeps the first maximum
-    }
-  }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    csum += __shfl_xor_sync(0xffffffffu, csum, o);
-    ArgMax b2;
-    b2.v = __shfl_xor_sync(0xffffffffu, am.v, o);
-    b2.i = __shfl_xor_sync(0xffffffffu, am.i, o);
-    am = better(am, b2);
-  }
-  const unsigned any_bad = __ballot_sync(0xffffffffu, bad);
-  if (lane == 0) {
-    sh.wc[w] = csum;
-    sh.wa[w] = am;
-    sh.wscan[w] = any_bad ? 1u : 0u;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long tc = 0;
-    ArgMax ta{-INFINITY, 0x7fffffff};
-    uint32_t tbad = 0;
-    for (int i = 0; i < Sh::kNW; ++i) {
-      tc += sh.wc[i];
-      ta = better(ta, sh.wa[i]);
-      tbad |= sh.wscan[i];
-    }
-    sh.cl_csum = tc;
-    sh.cl_arg = ta;
-    sh.cl_bad = tbad;
-  }
-  cl.sync();
-  QuantResult r{0, -1, false};
-  unsigned long long total = 0;
-  ArgMax g{-INFINITY, 0x7fffffff};
-  for (int q = 0; q < CL; ++q) {
-    const Sh* o = cl.map_shared_rank(&sh, q);
-    total += o->cl_csum;
-    g = better(g, o->cl_arg);
-    r.bad |= o->cl_bad != 0;
-  }
-  r.resid = (long long)T - (long long)total;
-  r.argmax = g.i;
-#pragma unroll
-  for (int i = 0; i < E; ++i) {
-    if (v0 + i == g.i) {
-      const long long ci = (long long)c[i] + r.resid;
-      if (ci < (long long)floor_c || ci > (long long)T) r.bad = true;
-      c[i] = (uint32_t)ci;
-    }
-  }
-  return r;
-}
-
-// Exclusive prefix sum of the final counts into cdf_row.
-template <int E, typename Sh>
-__device__ void scan_round(const uint32_t (&c)[E], int v0, int V, uint32_t T, uint32_t* cdf_row,
-                           cg::cluster_group& cl, Sh& sh) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  uint32_t local[E];
-  uint32_t run = 0;
-#pragma unroll
-  for (int i = 0; i < E; ++i) {
-    local[i] = run;
-    run += c[i];
-  }
-  uint32_t inc = run;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += t;
-  }
-  __syncthreads();                                 // wscan was read by the quantiser round
-  if (lane == 31) sh.wscan[w] = inc;
-  __syncthreads();
-  uint32_t before = 0, total = 0;
-  for (int i = 0; i < Sh::kNW; ++i) {
-    if (i < w) before += sh.wscan[i];
-    total += sh.wscan[i];
-  }
-  if (threadIdx.x == 0) sh.cl_total = total;
-  cl.sync();
-  uint32_t off = 0;
-  for (int r = 0; r < (int)cl.block_rank(); ++r) off += cl.map_shared_rank(&sh, r)->cl_total;
-  const uint32_t base = off + before + inc - run;
-#pragma unroll
-  for (int i = 0; i < E; ++i)
-    if (v0 + i < V) cdf_row[v0 + i] = base + local[i];
-  if (v0 <= V - 1 && V - 1 < v0 + E) cdf_row[V] = T;
 }
 
 // ======================================================================= step
@@ -1732,23 +1562,165 @@ __global__ void k_prepare_prefill(Batch b, int n_streams, int m, int V, const in
   }
 }
 
-// Standalone quantiser over rows of binary32 probabilities.
-template <int E>
-__global__ void __cluster_dims__(kVocabCluster, 1, 1) __launch_bounds__(kVocabThreads)
-    k_probs_to_cdf(const float* p, int V, int log2T, uint32_t floor_c, uint32_t* cdf,
-                   int32_t* status) {
-  __shared__ VocabShared sh;
+// Standalone quantiser over rows of binary32 probabilities: a cluster of
+// kP2cCtas CTAs per row, warp gw of its 32 owning the 128 IT symbols from
+// 128 IT gw, in IT pieces of 128 (four consecutive symbols per lane), so that
+// loads and stores are whole lines.  The counts stay in registers; the row's
+// sum, first maximum and bad flag and the counts before each warp take one
+// exchange (every warp's partial into every CTA's inbox, one cluster barrier),
+// then each warp scans its own pieces.  A row of the CDF has V + 1 entries, so
+// rows start at any of the four offsets of a 16-byte vector: lanes pass their
+// last entries on and store aligned vectors.
+// Bound by memory.  The first version (eight CTAs of 512 threads, 12
+// consecutive symbols per thread, block and cluster rounds of 64-bit shuffles
+// and three cluster barriers) took 117 us for 256 rows of 49,152 (100 MB).
+constexpr int kP2cCtas = 4, kP2cThreads = 256;
+constexpr int kP2cWarps = kP2cCtas * kP2cThreads / 32;     // 32: one inbox entry per lane
+struct P2cPart {
+  unsigned long long sum;     // counts of the warp
+  uint32_t v;                 // its first maximum's value bits (p >= 0 orders as unsigned)
+  int32_t i;                  // and index
+  uint32_t bad;
+  uint32_t pad[3];
+};
+
+__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// The first maximum over the warp of (value bits, index).
+__device__ __forceinline__ void warp_first_max(uint32_t& v, int32_t& i) {
+  const uint32_t m = __reduce_max_sync(0xffffffffu, v);
+  i = __reduce_min_sync(0xffffffffu, v == m ? i : 0x7fffffff);
+  v = m;
+}
+
+template <int IT>
+__global__ void __cluster_dims__(kP2cCtas, 1, 1) __launch_bounds__(kP2cThreads)
+    k_probs_to_cdf(const float* p, int V, int log2T, uint32_t floor_c, uint32_t* cdf, int32_t* status,
+                   int per_row) {
+  __shared__ P2cPart inbox[kP2cWarps];
   cg::cluster_group cl = cg::this_cluster();
-  const int j = blockIdx.x / kVocabCluster;
-  const int rank = (int)cl.block_rank();
-  const int v0 = rank * kVocabThreads * E + threadIdx.x * E;
-  float pr[E];
-  load_run<E>(p + (size_t)j * V, v0, V, pr, 0.f);
-  uint32_t c[E];
-  const QuantResult q = quantise_round<E, kVocabCluster>(pr, v0, V, log2T, floor_c, c, cl, sh);
-  if (q.bad && threadIdx.x == 0 && rank == 0) atomicOr(status + j, ST_NUMERIC);
-  scan_round<E>(c, v0, V, 1u << log2T, cdf + (size_t)j * (V + 1), cl, sh);
+  const int j = blockIdx.x / kP2cCtas, rank = (int)cl.block_rank();
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, gw = rank * (kP2cThreads / 32) + w;
+  const int vw = gw * 128 * IT;                    // the warp's first symbol
+  // every CTA must have started before its inbox is written
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  const uint32_t T = 1u << log2T, K = T - (uint32_t)V * floor_c;
+  const float Kf = (float)K;
+  const float* row = p + (size_t)j * V;
+  float x[IT][4];
+  const bool vec = (reinterpret_cast<uintptr_t>(row) & 15) == 0;
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int v = vw + it * 128 + lane * 4;
+    if (vec && v + 4 <= V) {
+      const float4 u = __ldcs(reinterpret_cast<const float4*>(row + v));
+      x[it][0] = u.x;
+      x[it][1] = u.y;
+      x[it][2] = u.z;
+      x[it][3] = u.w;
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) x[it][q] = v + q < V ? row[v + q] : 0.f;
+    }
+  }
+  uint32_t c[IT][4], ts = 0, am_v = 0, am_c = 0;   // ts: at most 64 counts below 2^25
+  int32_t am_i = 0x7fffffff;
+  bool bad = false;
+  float best = -INFINITY;
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int v = vw + it * 128 + lane * 4 + q;
+      c[it][q] = 0;
+      if (v < V) {
+        const uint32_t n = floor_count(x[it][q], K, Kf, bad);
+        c[it][q] = n > floor_c ? n : floor_c;
+        ts += c[it][q];
+        if (x[it][q] > best) {                     // strict: keeps the first maximum
+          best = x[it][q];
+          am_i = v;
+          am_c = c[it][q];
+        }
+      }
+    }
+  }
+  am_v = best > 0.f ? __float_as_uint(best) : 0u;
+  const int32_t my_i = am_i;
+  P2cPart part;
+  part.sum = warp_sum_u64(ts);
+  warp_first_max(am_v, am_i);
+  part.v = am_v;
+  part.i = am_i;
+  part.bad = __any_sync(0xffffffffu, bad) ? 1u : 0u;
+  part.pad[0] = part.pad[1] = part.pad[2] = 0;
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  if (lane < kP2cCtas) cl.map_shared_rank(inbox, lane)[gw] = part;
   cl.sync();
+  const P2cPart o = inbox[lane];
+  const unsigned long long total = warp_sum_u64(o.sum);
+  uint32_t run = (uint32_t)warp_sum_u64(lane < gw ? o.sum : 0ull);
+  uint32_t gv = o.v;
+  int32_t gi = o.i;
+  warp_first_max(gv, gi);
+  const long long resid = (long long)T - (long long)total;
+  bool row_bad = __any_sync(0xffffffffu, o.bad != 0) && gw == 0 && lane == 0;
+  if (my_i == gi && my_i != 0x7fffffff) {          // the first maximum's final count stays within [floor, T]
+    const long long ci = (long long)am_c + resid;
+    row_bad |= ci < (long long)floor_c || ci > (long long)T;
+  }
+  if (row_bad) atomicOr(status + (per_row ? j : 0), ST_NUMERIC);
+  // exclusive prefix sum; the residual counts from the symbol after the maximum on
+  uint32_t* out = cdf + (size_t)j * (V + 1);
+  const int r = (int)((reinterpret_cast<uintptr_t>(out) >> 2) & 3);   // entry 0's place in its 16 bytes
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int v0 = vw + it * 128, v = v0 + lane * 4;
+    if (v0 >= V) break;                            // uniform across the warp
+    const uint32_t t4 = c[it][0] + c[it][1] + c[it][2] + c[it][3];
+    uint32_t inc = t4;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const uint32_t u = __shfl_up_sync(0xffffffffu, inc, s);
+      if (lane >= s) inc += u;
+    }
+    uint32_t e[4], at = run + inc - t4;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      e[q] = at + (gi < v + q ? (uint32_t)resid : 0u);
+      at += c[it][q];
+    }
+    run += __shfl_sync(0xffffffffu, inc, 31);
+    if (v0 + 128 <= V) {
+      const uint32_t p1 = __shfl_up_sync(0xffffffffu, e[1], 1), p2 = __shfl_up_sync(0xffffffffu, e[2], 1),
+                     p3 = __shfl_up_sync(0xffffffffu, e[3], 1);
+      uint4 u;
+      if (r == 0) u = make_uint4(e[0], e[1], e[2], e[3]);
+      else if (r == 1) u = make_uint4(p3, e[0], e[1], e[2]);
+      else if (r == 2) u = make_uint4(p2, p3, e[0], e[1]);
+      else u = make_uint4(p1, p2, p3, e[0]);
+      if (r == 0 || lane > 0) {
+        __stcs(reinterpret_cast<uint4*>(out + v - r), u);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q < 4 - r) out[v + q] = e[q];
+      }
+      if (lane == 31) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q >= 4 - r) out[v + q] = e[q];
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (v + q < V) out[v + q] = e[q];
+    }
+  }
+  if (gw == 0 && lane == 0) out[V] = T;
 }
 
 __global__ void k_floor_counts(const float* p, int64_t n, uint32_t K, uint32_t floor_c,
@@ -1761,34 +1733,101 @@ __global__ void k_floor_counts(const float* p, int64_t n, uint32_t K, uint32_t f
   }
 }
 
-// Mixed-distribution NLL forward / backward, one CTA per row.
-__global__ void __launch_bounds__(kVocabThreads)
+// Mixed-distribution NLL forward / backward, one CTA of NT threads per row.
+//
+// Bound by memory: the softmax's maximum and sum come from one pass (each
+// thread keeps a running maximum and rescales its sum when it rises), four
+// values a load where the rows allow it, so the forward reads z and b once
+// from HBM and the backward's second pass finds them in L2.  The first
+// version made a pass for the maximum and a pass for the sum, one value a
+// load: 113 us each way for 512 rows of 49,152 (201 MB in, backward 101 MB out).
+constexpr int kNllVec = 4;                         // vectors of four in flight per array
+
+// fn(v, z_v, b_v) for the row's symbols in steps of the block; `vec`: 16-byte
+// aligned rows.
+template <int NT, typename F>
+__device__ __forceinline__ void nll_pass(const float* zr, const float* br, int V, bool vec, F fn) {
+  int done = 0;
+  if (vec) {
+    const int nv = V / 4;
+    for (int q0 = threadIdx.x; q0 < nv; q0 += NT * kNllVec) {
+      float4 zv[kNllVec], bv[kNllVec];
+#pragma unroll
+      for (int k = 0; k < kNllVec; ++k)
+        if (q0 + NT * k < nv) {
+          zv[k] = __ldg(reinterpret_cast<const float4*>(zr) + q0 + NT * k);
+          bv[k] = __ldg(reinterpret_cast<const float4*>(br) + q0 + NT * k);
+        }
+#pragma unroll
+      for (int k = 0; k < kNllVec; ++k)
+        if (q0 + NT * k < nv) fn(4 * (q0 + NT * k), zv[k], bv[k], 4);
+    }
+    done = 4 * nv;
+  }
+  for (int v = done + threadIdx.x; v < V; v += NT)
+    fn(v, make_float4(zr[v], 0.f, 0.f, 0.f), make_float4(br[v], 0.f, 0.f, 0.f), 1);
+}
+
+template <int NT>
+__global__ void __launch_bounds__(NT)
     k_mix_nll(const float* z, const float* bv, const float* png, const float* theta,
               const int32_t* target, const int32_t* warm, const float* gout, int V, float tau,
               float* loss, float* db, float* dth) {
-  __shared__ VocabShared sh;
+  __shared__ float2 part[NT / 32];
   const int j = blockIdx.x;
   const float* zr = z + (size_t)j * V;
   const float* br = bv + (size_t)j * V;
+  float* dr = db ? db + (size_t)j * V : nullptr;
   const int t = target[j];
   if (t < 0 || t >= V) {     // out-of-range target: NaN loss and gradients
-    for (int v = threadIdx.x; v < V && db; v += kVocabThreads) db[(size_t)j * V + v] = NAN;
+    for (int v = threadIdx.x; v < V && dr; v += NT) dr[v] = NAN;
     if (threadIdx.x == 0) {
       if (loss) loss[j] = NAN;
       if (dth) dth[2 * j] = dth[2 * j + 1] = NAN;
     }
     return;
   }
+  const bool vec = ((reinterpret_cast<uintptr_t>(zr) | reinterpret_cast<uintptr_t>(br) |
+                     reinterpret_cast<uintptr_t>(dr)) & 15) == 0;
   // s = z / tau + b as the coding step forms it (Sec. 3.2, Sec. 3.6): one
   // fused multiply-add by the rounded reciprocal of tau
   const float inv_tau = 1.0f / tau;
-  float mx = -INFINITY;
-  for (int v = threadIdx.x; v < V; v += kVocabThreads) mx = fmaxf(mx, __fmaf_rn(zr[v], inv_tau, br[v]));
-  const float M = block_max(mx, sh);
-  float ls = 0.f;
-  for (int v = threadIdx.x; v < V; v += kVocabThreads) ls += expf(__fmaf_rn(zr[v], inv_tau, br[v]) - M);
-  const float S = block_sum(ls, sh);
-  const float pts = __fdiv_rn(expf(__fmaf_rn(zr[t], inv_tau, br[t]) - M), S);
+  auto score = [&](float zz, float bb) { return __fmaf_rn(zz, inv_tau, bb); };
+  float m = -INFINITY, ls = 0.f;
+  // (m, ls) <- merged with another maximum and sum; while a maximum is -inf
+  // its sum is 0, or NaN if a NaN was seen
+  auto add = [&](float mx, float sum) {
+    if (mx > m) {
+      ls = (m == -INFINITY ? ls : ls * expf(m - mx)) + sum;
+      m = mx;
+    } else {
+      ls += mx == m || mx == -INFINITY ? sum : sum * expf(mx - m);
+    }
+  };
+  nll_pass<NT>(zr, br, V, vec, [&](int, float4 a, float4 b, int n) {
+    const float s0 = score(a.x, b.x);
+    if (n == 1) {                                  // exp(s0 - s0): 1, or NaN for an infinite or NaN score
+      add(s0, s0 == -INFINITY ? 0.f : expf(s0 - s0));
+      return;
+    }
+    const float s1 = score(a.y, b.y), s2 = score(a.z, b.z), s3 = score(a.w, b.w);
+    const float mx = fmaxf(fmaxf(s0, s1), fmaxf(s2, s3));
+    if (mx > m) {
+      if (m > -INFINITY) ls *= expf(m - mx);
+      m = mx;
+    }
+    if (m > -INFINITY) ls += (expf(s0 - m) + expf(s1 - m)) + (expf(s2 - m) + expf(s3 - m));
+    else if (s0 != s0 || s1 != s1 || s2 != s2 || s3 != s3) ls = NAN;
+  });
+#pragma unroll
+  for (int o = 16; o; o >>= 1) add(__shfl_xor_sync(0xffffffffu, m, o), __shfl_xor_sync(0xffffffffu, ls, o));
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_float2(m, ls);
+  __syncthreads();
+  m = part[0].x;
+  ls = part[0].y;
+  for (int i = 1; i < NT / 32; ++i) add(part[i].x, part[i].y);
+  const float M = m, S = m == -INFINITY ? NAN : ls;
+  const float pts = __fdiv_rn(expf(score(zr[t], br[t]) - M), S);
   const float pngs = png[(size_t)j * V + t];
   const float th0 = theta[2 * j], th1 = theta[2 * j + 1];
   const float tm = fmaxf(th0, th1);
@@ -1798,12 +1837,19 @@ __global__ void __launch_bounds__(kVocabThreads)
   const float pm = wu ? pts : w0 * pts + w1 * pngs;
   const float g = gout ? gout[j] : 1.f;
   if (loss && threadIdx.x == 0) loss[j] = -logf(pm);
-  if (db) {
+  if (dr) {
     const float rho = wu ? 1.f : w0 * pts / pm;
-    for (int v = threadIdx.x; v < V; v += kVocabThreads) {
-      const float ptv = __fdiv_rn(expf(__fmaf_rn(zr[v], inv_tau, br[v]) - M), S);
-      db[(size_t)j * V + v] = g * rho * (ptv - (v == t ? 1.f : 0.f));
-    }
+    auto grad = [&](float zz, float bb, int v) {
+      const float ptv = __fdiv_rn(expf(score(zz, bb) - M), S);
+      return g * rho * (ptv - (v == t ? 1.f : 0.f));
+    };
+    nll_pass<NT>(zr, br, V, vec, [&](int v, float4 a, float4 b, int n) {
+      if (n == 1)
+        dr[v] = grad(a.x, b.x, v);
+      else
+        __stcs(reinterpret_cast<float4*>(dr + v), make_float4(grad(a.x, b.x, v), grad(a.y, b.y, v + 1),
+                                                              grad(a.z, b.z, v + 2), grad(a.w, b.w, v + 3)));
+    });
   }
   if (dth && threadIdx.x == 0) {
     dth[2 * j] = wu ? 0.f : g * (w0 - w0 * pts / pm);
@@ -1868,7 +1914,7 @@ __global__ void k_search(Batch b, int V, const uint32_t* cdf, const uint32_t* ta
 }  // namespace
 
 // Elements per thread for a vocabulary of V over `ctas` CTAs of `threads`.
-static int vocab_E(int V, int ctas = kVocabCluster, int threads = kVocabThreads) {
+static int vocab_E(int V, int ctas, int threads) {
   const int per = ctas * threads;
   int e = (V + per - 1) / per;
   e = (e + 3) / 4 * 4;
@@ -2034,21 +2080,20 @@ cudaError_t launch_prepare_prefill(const Batch& b, int n_streams, int m, int V, 
                        offs, lens, f_slots, f_pos, f_tok, nB_fwd, obs_step, nb_step, z_idx);
 }
 
-template <int E>
-static cudaError_t p2c_t(const float* p, int n, int V, int log2T, uint32_t floor_c, uint32_t* cdf,
-                         int32_t* status, cudaStream_t s) {
-  k_probs_to_cdf<E><<<n * kVocabCluster, kVocabThreads, 0, s>>>(p, V, log2T, floor_c, cdf, status);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_probs_to_cdf(const float* p, int n, int V, int log2T, uint32_t floor_c,
-                                uint32_t* cdf, int32_t* status, cudaStream_t s) {
-  switch (vocab_E(V)) {
-    case 4: return p2c_t<4>(p, n, V, log2T, floor_c, cdf, status, s);
-    case 8: return p2c_t<8>(p, n, V, log2T, floor_c, cdf, status, s);
-    case 12: return p2c_t<12>(p, n, V, log2T, floor_c, cdf, status, s);
-    case 16: return p2c_t<16>(p, n, V, log2T, floor_c, cdf, status, s);
-  }
+cudaError_t launch_probs_to_cdf(const float* p, int n, int V, int log2T, uint32_t floor_c, uint32_t* cdf,
+                                int32_t* status, bool per_row, cudaStream_t s) {
+  // pieces of 128 symbols per warp, in powers of two but for the full vocabulary's 12
+  const int it = (V + 128 * kP2cWarps - 1) / (128 * kP2cWarps);
+  auto go = [&](auto kern) {
+    kern<<<n * kP2cCtas, kP2cThreads, 0, s>>>(p, V, log2T, floor_c, cdf, status, per_row);
+    return cudaGetLastError();
+  };
+  if (it <= 1) return go(k_probs_to_cdf<1>);
+  if (it <= 2) return go(k_probs_to_cdf<2>);
+  if (it <= 4) return go(k_probs_to_cdf<4>);
+  if (it <= 8) return go(k_probs_to_cdf<8>);
+  if (it <= 12) return go(k_probs_to_cdf<12>);
+  if (it <= 16) return go(k_probs_to_cdf<16>);
   return cudaErrorInvalidValue;
 }
 
@@ -2082,7 +2127,11 @@ cudaError_t launch_mix_nll(const float* z, const float* b, const float* png, con
                            const int32_t* target, const int32_t* warm, const float* gout, int n,
                            int V, float tau, float* loss, float* db, float* dtheta,
                            cudaStream_t s) {
-  k_mix_nll<<<n, kVocabThreads, 0, s>>>(z, b, png, theta, target, warm, gout, V, tau, loss, db, dtheta);
+  // few rows: more threads per row; many: two CTAs per SM
+  if (n <= 152)
+    k_mix_nll<1024><<<n, 1024, 0, s>>>(z, b, png, theta, target, warm, gout, V, tau, loss, db, dtheta);
+  else
+    k_mix_nll<512><<<n, 512, 0, s>>>(z, b, png, theta, target, warm, gout, V, tau, loss, db, dtheta);
   return cudaGetLastError();
 }
 

@@ -87,7 +87,7 @@ extern "C" int nc_probs_to_cdf_noalloc(const float* p, int n, int V, int log2_to
   int32_t hs[NC_NOALLOC_MAX_ROWS];
   // the words keep the previous call's values: clear the ones this call uses
   if (cudaMemsetAsync(status, 0, (size_t)n * sizeof(int32_t), s) != cudaSuccess ||
-      nc::launch_probs_to_cdf(p, n, V, log2_total, floor_c, cdf, status, s) != cudaSuccess ||
+      nc::launch_probs_to_cdf(p, n, V, log2_total, floor_c, cdf, status, true, s) != cudaSuccess ||
       cudaMemcpyAsync(hs, status, (size_t)n * sizeof(int32_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return NC_ECUDA;
