@@ -29,9 +29,9 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 __device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
 }
 
 // floor(p * K) for a binary32 p in [0, 2) and K < 2^24, exactly: p = m 2^(e-150)
@@ -156,24 +156,22 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // e^x = 2^(x log2 e) for the few scalar exponentials of a step.
 __device__ __forceinline__ float exp_fast(float x) { return ex2_approx(__fmul_rn(x, kLog2e)); }
 
-// Every CTA's inbox for one exchange (two alternate): each warp of the
-// cluster stores its partials at its global index gw in every CTA's inbox,
-// as posted remote stores made visible by a cluster barrier's release (the
-// step kernel) or as asynchronous remote stores that complete their bytes on
-// the receiving CTA's mbarrier (the prefill loop), so that afterwards every
-// warp reduces them from its own CTA's shared memory.
+// Every CTA's inbox for one exchange of the step kernel (two alternate): each
+// warp of the cluster stores its partials at its global index gw in every
+// CTA's inbox, as posted remote stores made visible by a cluster barrier's
+// release, so that afterwards every warp reduces them from its own CTA's
+// shared memory.
 struct StepSlot {
   float4 sm[kClusterWarps];   // softmax: warp maximum m_w, sum of exp(s - m_w), entropy part
   uint4 qn[kClusterWarps];    // quantiser: count sum, first maximum (value bits, index), bad flag
   float4 obs;                             // the observed token's p_tilde(t), p_ng(t), log p_tilde(t)
 };
 
-constexpr int kSnapBufs = 3;   // N-gram states in flight in the prefill loop
+constexpr int kSnapBufs = 4;   // N-gram states in flight in the prefill loop
 constexpr int kSeqMax = 1024;  // positions of one prefill chunk at most (a power of two dividing C < L <= 2,048)
 struct StepShared {
   StepSlot slot[2];
-  NgSnap ng[kSnapBufs];
-  uint64_t xbar[2];           // the prefill loop's exchange rounds, by slot
+  NgSnap ng;
 };
 
 // This thread's place in the cluster's split of the vocabulary.
@@ -229,9 +227,7 @@ __device__ __forceinline__ void push_obs(cg::cluster_group& cl, float4* mine, fl
 // value goes to every CTA's inbox as an asynchronous remote store that
 // completes its bytes on that CTA's mbarrier of the round's slot; a CTA
 // arms its own mbarrier with the round's byte count and waits on it (acquire
-// at cluster scope).  Slot s serves rounds s, s + 2, ...: a sender reaches
-// round k + 2 only after every CTA's round k + 1 values, sent after each CTA
-// finished reading round k.
+// at cluster scope).
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t remote_addr(uint32_t a, int rank) {
   uint32_t r;
@@ -253,11 +249,6 @@ __device__ __forceinline__ uint4 as_u4(const T& v) {
 template <int CL, typename T>
 __device__ __forceinline__ void push_part_async(T* mine, const Lanes& L, T v, uint64_t* bar) {
   if (L.lane < CL) st_async16(remote_addr(smem_addr(mine + L.gw), L.lane), remote_addr(smem_addr(bar), L.lane), as_u4(v));
-}
-template <int CL>
-__device__ __forceinline__ void push_obs_async(float4* mine, float4 v, uint64_t* bar) {
-#pragma unroll
-  for (int r = 0; r < CL; ++r) st_async16(remote_addr(smem_addr(mine), r), remote_addr(smem_addr(bar), r), as_u4(v));
 }
 __device__ __forceinline__ void xbar_arm(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
@@ -284,10 +275,6 @@ __device__ __forceinline__ bool xbar_wait(uint64_t* bar, uint32_t parity) {
   }
   return false;
 }
-// Bytes of one round: the softmax partials and / or the quantiser partials
-// with the observed token's values.
-constexpr uint32_t kRoundSm = kClusterWarps * 16, kRoundQ = kClusterWarps * 16 + 16;
-
 // The inbox entries of global warps 4 lane .. 4 lane + 3.
 template <typename T>
 __device__ __forceinline__ void local_parts(const T* arr, int lane, T (&v)[4]) {
@@ -510,20 +497,14 @@ __device__ __forceinline__ uint4 quant_part(const float (&p)[E], const Lanes& L,
     excl = inc - ts;
     wsum = __shfl_sync(0xffffffffu, inc, 31);
   } else {
-    wsum = ts;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
+    wsum = __reduce_add_sync(0xffffffffu, ts);
   }
-  // first maximum: value bits (p >= 0 orders as unsigned) over the inverted index
-  unsigned long long key =
-      ((unsigned long long)(amv > 0.f ? __float_as_uint(amv) : 0u) << 32) | (uint32_t)~(uint32_t)am_i;
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, o);
-    key = k2 > key ? k2 : key;
-  }
+  // first maximum: value bits (p >= 0 orders as unsigned), then the lowest index
+  const uint32_t kv = amv > 0.f ? __float_as_uint(amv) : 0u;
+  const uint32_t hi = __reduce_max_sync(0xffffffffu, kv);
+  const uint32_t ix = __reduce_min_sync(0xffffffffu, kv == hi ? (uint32_t)am_i : 0xffffffffu);
   bad = __any_sync(0xffffffffu, bad) || wsum > kWarpCountCap;
-  return make_uint4(bad ? kWarpCountCap : wsum, (uint32_t)(key >> 32), ~(uint32_t)key, bad ? 1u : 0u);
+  return make_uint4(bad ? kWarpCountCap : wsum, hi, ix, bad ? 1u : 0u);
 }
 
 // The cluster's quantiser results: the residual T - sum c (added to the first
@@ -534,28 +515,26 @@ struct Quant {
   bool bad;
 };
 __device__ __forceinline__ Quant quant_reduce(const uint4 (&v)[4], const Lanes& L, uint32_t T) {
-  uint32_t tot = 0, off = 0;
-  unsigned long long key = 0;
+  uint32_t tot = 0, off = 0, kv = 0, ix = 0xffffffffu;
   bool bad = false;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < 4; ++i) {                    // the indexes rise with the warps
     tot += v[i].x;
     if (4 * L.lane + i < L.gw) off += v[i].x;
-    const unsigned long long k = ((unsigned long long)v[i].y << 32) | (uint32_t)~v[i].z;
-    key = k > key ? k : key;
+    if (i == 0 || v[i].y > kv) {
+      kv = v[i].y;
+      ix = v[i].z;
+    }
     bad |= v[i].w != 0u;
   }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    off += __shfl_xor_sync(0xffffffffu, off, o);
-    const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, key, o);
-    key = k2 > key ? k2 : key;
-  }
+  tot = __reduce_add_sync(0xffffffffu, tot);
+  off = __reduce_add_sync(0xffffffffu, off);
+  const uint32_t hi = __reduce_max_sync(0xffffffffu, kv);
+  ix = __reduce_min_sync(0xffffffffu, kv == hi ? ix : 0xffffffffu);
   Quant q;
   q.resid = (long long)T - (long long)tot;
   q.woff = (long long)off;
-  q.argmax = (int)~(uint32_t)key;
+  q.argmax = (int)ix;
   q.bad = __any_sync(0xffffffffu, bad);
   return q;
 }
@@ -639,6 +618,7 @@ __device__ __forceinline__ void cp_async16(void* dst_smem, const void* src) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_group1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
 // Copy one N-gram state into shared memory (asynchronously, 16 bytes per thread).
 __device__ __forceinline__ void snap_copy_async(NgSnap* dst, const NgSnap* src) {
@@ -688,7 +668,7 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1) k_vocab(Dims D, Batch b
   if (ngram) {
     load_counts<E>(st.uni, L.v0, V, cnt);
     zero_region<E>(spw, L.lane);
-    ng_snapshot(D, st, &sh.ng[0], threadIdx.x, step_threads<CL>());
+    ng_snapshot(D, st, &sh.ng, threadIdx.x, step_threads<CL>());
     __syncthreads();
   }
   const int i_tok = st.n_coded + 1;              // 1-based index of the token being coded
@@ -713,7 +693,7 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1) k_vocab(Dims D, Batch b
   // ---- softmax (Sec. 3.6) and the N-gram distribution
   float png[E];
   if (ngram) {
-    ngram_probs<E, FULL>(sh.ng[0], spw, L, V, cnt, png);
+    ngram_probs<E, FULL>(sh.ng, spw, L, V, cnt, png);
     if (probe && io.probe_png) store_run<E>(io.probe_png + prow, L.v0, V, png);
   } else {
 #pragma unroll
@@ -804,33 +784,60 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1) k_vocab(Dims D, Batch b
 }
 
 // The vocabulary passes of a prefill chunk (encoder): the cluster of stream
-// row j runs its positions r = 0 .. m - 1 in order while j < nb_step[r],
-// with the bias, the unigram counts, the mixer's log-weights and the position
-// kept on chip and the N-gram state of each prediction read from snap (made
-// ahead by k_ngram_seq).  Under the log-loss mixer the head's step does not
-// wait for the mixer, so position r's quantiser and mixer results share the
-// exchange round of position r + 1's softmax: one round per position, with
-// no cluster barrier (each CTA waits on its own mbarrier for the round's
-// bytes).  The next position's logits, token and activity and the N-gram
-// state two positions ahead are fetched while the round's values travel.
+// row j runs its positions r = 0 .. R - 1 in order (R: the chunk's positions
+// the stream still has), with the bias, the unigram counts, the mixer's
+// log-weights and the position kept on chip and the N-gram state of each
+// prediction read from snap (made ahead by k_ngram_seq).
+//
+// One position's softmax needs the head's step of the one before, so the loop
+// is a serial chain: reduce the exchanged partials, p_tilde, the head's step,
+// the next scores, their partials, and the way to the other CTAs.  Only that
+// is on the chain.  Round r carries position r's softmax partials and the
+// values of its observed token (its numerator and warp maximum, from which
+// every thread forms p_tilde(t) as the owner does, its score and p_ng(t)), so
+// the mixed-NLL step needs no round of its own.  While round r travels
+// (a window of about 1 us), each warp
+//   - fetches position r + 1's logits and adds its N-gram masses;
+//   - codes position r - 1 (mix, counts, its partials into the slot of round
+//     r + 1) and takes its mixer step;
+//   - finishes position r - 3 (residual, interval) from the partials that came
+//     with round r - 1.
+// Four slots: what is in slot k is read by the end of window k + 1, before the
+// warp sends its round k + 2; a sender writes slot k again in window k + 3 at
+// the earliest, after every warp's round k + 2.
+//
+// Measured (GB300, one stream of 8,192 tokens, 16 CTAs): 3.1 us a position when
+// coding a position came before the next one's partials, 2.4 us now.
+constexpr int kSeqSlots = 4;
+constexpr uint32_t kRoundPart = kClusterWarps * 16;        // bytes of one array of warp partials
+struct SeqShared {
+  struct Slot {
+    float4 sm[kClusterWarps];   // softmax: warp maximum m_w, sum of exp(s - m_w), entropy part
+    uint4 qn[kClusterWarps];    // quantiser partials of the position two back
+    float4 obs;                 // the observed token's numerator, warp maximum, score, p_ng
+  } slot[kSeqSlots];
+  NgSnap ng[kSnapBufs];         // N-gram states of the positions ahead
+  uint64_t xbar[kSeqSlots];     // the rounds' barriers
+  int32_t obs[kSeqMax], nb[kSeqMax];   // the chunk's tokens and active rows, per position
+};
+
 template <int E, bool FULL, int CL>
 __global__ void __launch_bounds__(step_threads<CL>(), 1)
     k_vocab_seq(Dims D, Batch b, VocabIO io, int m, int n_streams, const float* zrows, const int32_t* nb_step,
                 const int32_t* obs_step, const NgSnap* snap) {
   extern __shared__ float4 dyn4[];
-  __shared__ StepShared sh;
-  __shared__ int32_t s_obs[kSeqMax], s_nb[kSeqMax];   // the chunk's tokens and active rows, per position
+  __shared__ SeqShared sh;
   cg::cluster_group cl = cg::this_cluster();
   const int j = blockIdx.x / CL;
   pdl_wait();
   pdl_trigger();
   if (m < 1 || j >= nb_step[0]) return;          // uniform across the cluster
   for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    s_obs[i] = obs_step[(size_t)i * n_streams + j];
-    s_nb[i] = nb_step[i];
+    sh.obs[i] = obs_step[(size_t)i * n_streams + j];
+    sh.nb[i] = nb_step[i];
   }
   if (threadIdx.x == 0) {
-    for (int k = 0; k < 2; ++k)
+    for (int k = 0; k < kSeqSlots; ++k)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&sh.xbar[k])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -838,11 +845,13 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1)
   StreamDev& st = b.st[b.slots[j]];
   const int V = D.V;
   const bool ngram = D.order > 0;
-  const bool fused = D.rule != NC_RULE_MIXED_NLL;
+  const bool nll = D.rule == NC_RULE_MIXED_NLL;
   const float inv_tau = 1.0f / D.tau;
   const uint32_t T = 1u << D.log2T, K = T - (uint32_t)V * D.floor;
   const float Kf = (float)K;
-  float* spw = reinterpret_cast<float*>(dyn4) + L.w * 32 * E;
+  // the warp's slot masses of even and odd positions
+  float* spw0 = reinterpret_cast<float*>(dyn4) + L.w * 64 * E;
+  auto spw = [&](int q) { return spw0 + (q & 1) * (32 * E); };
   const float* zj = zrows + (size_t)b.z_idx[j] * V;
   const NgSnap* gj = ngram ? snap + b.z_idx[j] : nullptr;
 
@@ -855,182 +864,206 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1)
     for (int i = 0; i < E; ++i) bias[i] = 0.f;
   }
   __syncthreads();                               // the tokens and active rows are in shared memory
-  bool act1 = 1 < m && j < s_nb[1];              // positions r + 1 and r + 2 exist
-  bool act2 = act1 && 2 < m && j < s_nb[2];
+  int R = 1;                                     // positions: the active rows only fall
+  for (int hi = m; R < hi;) {
+    const int mid = (R + hi + 1) >> 1;
+    if (j < sh.nb[mid - 1]) R = mid;
+    else hi = mid - 1;
+  }
   if (ngram) {
     load_counts<E>(st.uni, L.v0, V, cnt);
-    zero_region<E>(spw, L.lane);
-    snap_copy_async(&sh.ng[0], gj);
-    if (act1) snap_copy_async(&sh.ng[1], gj + 1);
-    if (act2) snap_copy_async(&sh.ng[2], gj + 2);
+    zero_region<E>(spw(0), L.lane);
+    zero_region<E>(spw(1), L.lane);
+    for (int i = 0; i < kSnapBufs && i < R; ++i) snap_copy_async(&sh.ng[i], gj + i);
   } else {
 #pragma unroll
     for (int i = 0; i < E; ++i) cnt[i] = 0;
   }
   load_runf<E, FULL>(zj, L.v0, V, z, -INFINITY);
-  int t = s_obs[0];
   float th0 = st.theta[0], th1 = st.theta[1];
   const int n0 = st.n_coded;
+  float last_pts = st.pt_obs, last_pngs = st.png_obs;
   if (ngram) cp_async_wait_all();
   cl.sync();                                     // the first N-gram states are in shared memory, every
                                                  // CTA's exchange barriers initialised
-  if (ngram) ngram_scatter<E>(sh.ng[0], spw, L);
 
-  // the previous position's values its quantiser and mixer step need
-  bool pend = false, p_skip = false, p_mix = false, p_own = false;
-  int p_t = 0, p_pos = 0, p_am_i = 0x7fffffff;
-  uint32_t p_below = 0, p_ct = 0, p_am_c = 0;
-  float2 p_w = make_float2(0.f, 0.f);
-  float last_pts = st.pt_obs, last_pngs = st.png_obs;
-  int nb = 0;                                    // exchange rounds taken
-  bool xok = true;                               // no exchange wait has given up
-  int r = 0, t_last = -1;
-
-  // interval, numeric checks and mixer step of the pending position from its
-  // inbox `slot`
-  auto finish = [&](const StepSlot& slot, const float (&pt)[E], bool with_head) {
-    uint4 qv[4];
-    local_parts(slot.qn, L.lane, qv);
-    const Quant q = quant_reduce(qv, L, T);
-    const float4 o = slot.obs;
-    if (p_own)
-      write_interval(io.intervals + 2 * ((size_t)j * io.interval_stride + p_pos), q, p_t, p_below, p_ct);
-    if ((q.bad && L.rank == 0 && threadIdx.x == 0) || final_count_bad(q, p_am_i, p_am_c, D.floor, T))
-      atomicOr(&st.status, ST_NUMERIC);
-    if (!p_skip) {
-      float scale;
-      mixer_update(D, p_mix, p_w, o.x, o.y, o.z, th0, th1, scale);
-      if (with_head && D.use_head)
-        head_update<E>(bias, pt, __fmul_rn(D.alpha, scale), L.v0, p_t, p_t >= L.v0 && p_t < L.v0 + E);
-      last_pts = o.x;
-      last_pngs = o.y;
+  // the warp's entropy part of the prediction whose masses are in `sp`, its
+  // counts those of cnt and, once more, token `more` (Sec. 3.7)
+  auto entropy = [&](const float* sp, float cu, int more) {
+    float h = 0.f;
+#pragma unroll
+    for (int i = 0; i < E; ++i) {
+      if (in_vocab<FULL>(L.v0 + i, V)) {
+        const float p = __fmaf_rn(cu, (float)(cnt[i] + 1 + (L.v0 + i == more ? 1 : 0)), sp[L.lane * E + i]);
+        if (p > 0.f) h = __fmaf_rn(-p, log2f(p), h);
+      }
     }
+    return h;
   };
 
-  bool live = true;
-  while (live) {
-    if (t < 0 || t >= V) {                       // rejected on the host; never index with it
-      if (L.rank == 0 && threadIdx.x == 0) atomicOr(&st.status, ST_BAD_TOKEN);
-      break;                                     // uniform across the cluster
-    }
-    const bool more = act1;
-    // probes at the stream's probe_tok-th token (uniform across the cluster)
-    const bool probe = io.probe_tok == (int64_t)(n0 + r + 1);
-    const size_t prow = (size_t)(io.probe_row ? io.probe_row[j] : j) * V;
-    if (probe && io.probe_z) store_run<E>(io.probe_z + prow, L.v0, V, z);
+  // coded positions not yet finished: [0] the last one coded, [1], [2] before it
+  struct Pend {
+    int t, pos, am_i;
+    uint32_t below, ct, am_c;
+    bool own;
+  } pend[3];
+  // the position before the current one, not yet coded
+  float pt[E];
+  Soft sm{0.f, 0.f, 0.f};
+  float2 w = mix_weights(th0, th1);              // the weights of the position to be coded next
+  float cu = 0.f, cu_next = 0.f, h = 0.f;
+  int t_prev = -1;
+  bool skipped = false, mixing = false;
+  bool xok = true;                               // no exchange wait has given up
+  int r = 0;
 
-    // ---- softmax partials of position r (its slot masses are in spw)
+  // the observed token's p_tilde, p_ng and log p_tilde at the position whose
+  // exchange is (o, sm): the owner's arithmetic
+  auto obs_step_mixer = [&](const float4& o, float& scale) {
+    const float f = o.y == -INFINITY ? 0.f : __fdividef(exp_fast(__fsub_rn(o.y, sm.M)), sm.S);
+    const float pts = __fmul_rn(o.x, f);
+    mixer_update(D, mixing, w, pts, o.w, __fsub_rn(__fsub_rn(o.z, sm.M), __logf(sm.S)), th0, th1, scale);
+    last_pts = pts;
+    last_pngs = o.w;
+  };
+  // code position q = r - 1: the mix, its counts and their partials into the
+  // slot of round q + 2; then its mixer step and counts
+  auto code = [&](int q) {
+    const size_t prow = (size_t)(io.probe_row ? io.probe_row[j] : j) * V;
+    const bool probe = io.probe_tok == (int64_t)(n0 + q + 1);
     float png[E];
     if (ngram) {
-      ngram_read<E, FULL>(sh.ng[r % kSnapBufs].cu, spw, L, V, cnt, png);
+      ngram_read<E, FULL>(cu, spw(q), L, V, cnt, png);
     } else {
 #pragma unroll
       for (int i = 0; i < E; ++i) png[i] = 0.f;
     }
     if (probe && io.probe_png) store_run<E>(io.probe_png + prow, L.v0, V, png);
-    float s[E], e[E];
-    biased_logits<E, FULL>(z, bias, inv_tau, L.v0, V, s);
-    const bool owner = t >= L.v0 && t < L.v0 + E;
-    float s_t = 0.f, png_t = 0.f;
-    if (owner) {
-      s_t = pick<E>(s, L.v0, t);
-      png_t = pick<E>(png, L.v0, t);
-    }
-    const float4 part = softmax_part<E>(s, e, D.skip ? entropy_part<E>(png) : 0.f, D.skip != 0);
-    StepSlot& in = sh.slot[nb & 1];
-    uint64_t* xb = &sh.xbar[nb & 1];
-    push_part_async<CL>(in.sm, L, part, xb);
-    if (ngram) cp_async_wait_all();              // the state of position r + 2, added after this round
-    if (threadIdx.x == 0) xbar_arm(xb, kRoundSm + (pend ? kRoundQ : 0));
-    // while the round's values travel: position r + 1's logits, token and
-    // slot masses (its state arrived two rounds ago), the activity of r + 3
-    int t_n = 0;
-    bool act3 = false;
-    if (more) {
-      load_runf<E, FULL>(zj + (size_t)(r + 1) * V, L.v0, V, z, -INFINITY);
-      t_n = s_obs[r + 1];
-      act3 = act2 && r + 3 < m && j < s_nb[r + 3];
-      if (ngram) ngram_scatter<E>(sh.ng[(r + 1) % kSnapBufs], spw, L);
-    }
-    if (!__all_sync(0xffffffffu, xbar_wait(xb, (uint32_t)(nb >> 1) & 1u))) {
-      xok = false;
-      pend = false;
-      break;                                     // the other warps give up on their next round
-    }
-    // every warp of the cluster has added position r's masses (before its
-    // partials went out): its buffer takes the state of r + 3
-    if (ngram && act3) snap_copy_async(&sh.ng[(r + 3) % kSnapBufs], gj + r + 3);
-    ++nb;
-    float4 smv[4];
-    local_parts(in.sm, L.lane, smv);
-    const Soft sm = softmax_reduce(smv, D.skip != 0);
-    float pt[E];
-    if (pend) {                                  // position r - 1 (log-loss mixer: no head step here)
-      finish(in, pt, false);
-      pend = false;
-    }
-
-    // ---- position r: probabilities, counts, head step
-    const bool skipped = D.skip && sm.H < kSkipBits;
-    probs_tilde<E>(e, part.x, sm, pt);
-    const bool mixing = ngram && n0 + r + 1 > D.warmup;
-    const float2 w = mix_weights(th0, th1);
     float p[E];
     coded_probs<E>(pt, png, w, skipped, mixing, p);
-    if (probe && io.probe_pt) store_run<E>(io.probe_pt + prow, L.v0, V, pt);
     if (probe && io.probe_p) store_run<E>(io.probe_p + prow, L.v0, V, p);
-    StepSlot& nx = sh.slot[nb & 1];
-    if (owner)
-      push_obs_async<CL>(&nx.obs,
-                         make_float4(pick<E>(pt, L.v0, t), png_t, __fsub_rn(__fsub_rn(s_t, sm.M), __logf(sm.S)), 0.f),
-                         &sh.xbar[nb & 1]);
     uint32_t c[E], excl = 0;
-    const bool scan = io.intervals && t >= L.wbase && t < L.wbase + 32 * E;
-    const uint4 qp = quant_part<E, FULL>(p, L, V, K, Kf, D.floor, scan, finite_step(sm, w), c, excl, p_am_i, p_am_c);
-    push_part_async<CL>(nx.qn, L, qp, &sh.xbar[nb & 1]);
-    p_own = owner && io.intervals;
+    const bool here = t_prev >= L.wbase && t_prev < L.wbase + 32 * E;
+    const bool owner = t_prev >= L.v0 && t_prev < L.v0 + E;
+    pend[2] = pend[1];
+    pend[1] = pend[0];
+    Pend& n = pend[0];
+    const uint4 qp = quant_part<E, FULL>(p, L, V, K, Kf, D.floor, io.intervals && here, finite_step(sm, w), c, excl,
+                                         n.am_i, n.am_c);
+    push_part_async<CL>(sh.slot[(q + 2) & 3].qn, L, qp, &sh.xbar[(q + 2) & 3]);
+    n.own = owner && io.intervals;
+    n.t = t_prev;
+    n.pos = n0 + q;
     if (owner) {
-      counts_around<E>(c, L.v0, t, p_below, p_ct);
-      p_below += excl;
+      counts_around<E>(c, L.v0, t_prev, n.below, n.ct);
+      n.below += excl;
       if (ngram) {
 #pragma unroll
         for (int i = 0; i < E; ++i)
-          if (L.v0 + i == t) cnt[i] += 1;
+          if (L.v0 + i == t_prev) cnt[i] += 1;
       }
     }
-    p_t = t;
-    p_pos = n0 + r;                              // the token's index in its stream
-    p_skip = skipped;
-    p_mix = mixing;
-    p_w = w;
-    t_last = t;
-    if (fused) {
-      if (!skipped && D.use_head) head_update<E>(bias, pt, __fmul_rn(D.alpha, 1.f), L.v0, t, owner);
-      pend = true;
-    } else {
-      if (threadIdx.x == 0) xbar_arm(&sh.xbar[nb & 1], kRoundQ);
-      if (!__all_sync(0xffffffffu, xbar_wait(&sh.xbar[nb & 1], (uint32_t)(nb >> 1) & 1u))) {
-        xok = false;
-        break;
-      }
-      ++nb;
-      finish(nx, pt, true);
+    if (!nll && !skipped) {
+      float scale;
+      obs_step_mixer(sh.slot[q & 3].obs, scale);
     }
-    ++r;
-    t = t_n;
-    act1 = act2;
-    act2 = act3;
-    live = more;
+    w = mix_weights(th0, th1);
+  };
+  // interval and numeric checks of position q, pending as `n`, from the
+  // partials that came with round q + 2
+  auto finish = [&](int q, const Pend& n) {
+    uint4 qv[4];
+    local_parts(sh.slot[(q + 2) & 3].qn, L.lane, qv);
+    const Quant qr = quant_reduce(qv, L, T);
+    if (n.own)
+      write_interval(io.intervals + 2 * ((size_t)j * io.interval_stride + n.pos), qr, n.t, n.below, n.ct);
+    if ((qr.bad && L.rank == 0 && threadIdx.x == 0) || final_count_bad(qr, n.am_i, n.am_c, D.floor, T))
+      atomicOr(&st.status, ST_NUMERIC);
+  };
+  auto wait_round = [&](int k) {
+    xok = __all_sync(0xffffffffu, xbar_wait(&sh.xbar[k & 3], (uint32_t)(k >> 2) & 1u));
+    return xok;
+  };
+
+  if (ngram) {
+    ngram_scatter<E>(sh.ng[0], spw(0), L);
+    __syncwarp();
+    cu_next = sh.ng[0].cu;
+    if (D.skip) h = entropy(spw(0), cu_next, -1);
   }
-  if (pend) {
-    if (threadIdx.x == 0) xbar_arm(&sh.xbar[nb & 1], kRoundQ);
-    if (__all_sync(0xffffffffu, xbar_wait(&sh.xbar[nb & 1], (uint32_t)(nb >> 1) & 1u))) {
-      ++nb;
-      StepSlot& in = sh.slot[(nb - 1) & 1];
-      float none[E];
-      finish(in, none, false);
-    } else {
-      xok = false;
+  for (; r < R; ++r) {
+    const int t = sh.obs[r];
+    if (t < 0 || t >= V) {                       // rejected on the host; never index with it
+      if (L.rank == 0 && threadIdx.x == 0) atomicOr(&st.status, ST_BAD_TOKEN);
+      break;                                     // uniform across the cluster
+    }
+    // ---- the chain: position r's scores and partials
+    const bool probe = io.probe_tok == (int64_t)(n0 + r + 1);
+    const size_t prow = (size_t)(io.probe_row ? io.probe_row[j] : j) * V;
+    if (probe && io.probe_z) store_run<E>(io.probe_z + prow, L.v0, V, z);
+    float s[E], e[E];
+    biased_logits<E, FULL>(z, bias, inv_tau, L.v0, V, s);
+    const float4 part = softmax_part<E>(s, e, h, D.skip != 0);
+    if (ngram) cp_async_wait_group1();           // the state of position r + 2 has landed
+    SeqShared::Slot& in = sh.slot[r & 3];
+    uint64_t* xb = &sh.xbar[r & 3];
+    push_part_async<CL>(in.sm, L, part, xb);
+    if (threadIdx.x == 0) xbar_arm(xb, kRoundPart + 16 + (r >= 2 ? kRoundPart : 0));
+    if (t >= L.wbase && t < L.wbase + 32 * E) {  // the observed token's warp
+      float png_t = 0.f;
+      if (ngram && t >= L.v0 && t < L.v0 + E)    // counts up to position r - 2, and r - 1's token
+        png_t = __fmaf_rn(cu_next, (float)(pick<E>(cnt, L.v0, t) + 1 + (t == t_prev ? 1 : 0)), spw(r)[t - L.wbase]);
+      const int src = (t - L.wbase) / E;
+      const float4 o = make_float4(__shfl_sync(0xffffffffu, pick<E>(e, L.v0, t), src), part.x,
+                                   __shfl_sync(0xffffffffu, pick<E>(s, L.v0, t), src),
+                                   __shfl_sync(0xffffffffu, png_t, src));
+      if (L.lane < CL)
+        st_async16(remote_addr(smem_addr(&in.obs), L.lane), remote_addr(smem_addr(xb), L.lane), as_u4(o));
+    }
+    // ---- while the round travels
+    const bool more = r + 1 < R;
+    if (more) load_runf<E, FULL>(zj + (size_t)(r + 1) * V, L.v0, V, z, -INFINITY);
+    if (r >= 1) code(r - 1);
+    if (r >= 3) finish(r - 3, pend[2]);
+    cu = cu_next;
+    if (ngram && more) {
+      ngram_scatter<E>(sh.ng[(r + 1) % kSnapBufs], spw(r + 1), L);
+      __syncwarp();
+      cu_next = sh.ng[(r + 1) % kSnapBufs].cu;
+      if (D.skip) h = entropy(spw(r + 1), cu_next, t);
+    }
+    if (!wait_round(r)) break;                   // the other warps give up on their next round
+    // ---- the chain: position r's probabilities and head step
+    float4 smv[4];
+    local_parts(in.sm, L.lane, smv);
+    sm = softmax_reduce(smv, D.skip != 0);
+    skipped = D.skip && sm.H < kSkipBits;
+    mixing = ngram && n0 + r + 1 > D.warmup;
+    probs_tilde<E>(e, part.x, sm, pt);
+    float scale = 1.f;
+    if (nll && !skipped) obs_step_mixer(in.obs, scale);   // the head's step needs the mixer's
+    if (!skipped && D.use_head)
+      head_update<E>(bias, pt, __fmul_rn(D.alpha, scale), L.v0, t, t >= L.v0 && t < L.v0 + E);
+    if (probe && io.probe_pt) store_run<E>(io.probe_pt + prow, L.v0, V, pt);
+    // every warp of the CTA has added position r's masses (before its round
+    // went out): its buffer takes the state of r + kSnapBufs
+    if (ngram) {
+      if (r + kSnapBufs < R) snap_copy_async(&sh.ng[r % kSnapBufs], gj + r + kSnapBufs);
+      else cp_async_commit();
+    }
+    t_prev = t;
+  }
+  // ---- the last positions: code r - 1, finish r - 3, r - 2 and r - 1
+  if (r > 0 && xok) {
+    code(r - 1);
+    if (r >= 3) finish(r - 3, pend[2]);
+    if (r >= 2) {
+      if (threadIdx.x == 0) xbar_arm(&sh.xbar[r & 3], kRoundPart);
+      if (wait_round(r)) finish(r - 2, pend[1]);
+    }
+    if (xok) {
+      if (threadIdx.x == 0) xbar_arm(&sh.xbar[(r + 1) & 3], kRoundPart);
+      if (wait_round(r + 1)) finish(r - 1, pend[0]);
     }
   }
   if (!xok && L.lane == 0) atomicOr(&st.status, ST_TIMEOUT);
@@ -1052,7 +1085,7 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1)
     for (int a = start + D.L; a <= last; a += D.C) start += D.C;
     st.kv_start = start;
     st.n_coded = n0 + r;
-    st.last_tok = t_last;
+    st.last_tok = sh.obs[r - 1];
   }
 }
 
@@ -1957,7 +1990,7 @@ static cudaError_t prepare_vocab_tfc() {
   const int smem = step_threads<CL>() * E * (int)sizeof(float);
   cudaError_t e = cudaFuncSetAttribute(k_vocab<E, FULL, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_vocab_seq<E, FULL, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = cudaFuncSetAttribute(k_vocab_seq<E, FULL, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * smem);
   if (e == cudaSuccess && CL > 8) {
     e = cudaFuncSetAttribute(k_vocab<E, FULL, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess)
@@ -1971,7 +2004,7 @@ static bool clusters_fit() {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(CL);
   cfg.blockDim = dim3(step_threads<CL>());
-  cfg.dynamicSmemBytes = (size_t)step_threads<CL>() * E * sizeof(float);
+  cfg.dynamicSmemBytes = 2 * (size_t)step_threads<CL>() * E * sizeof(float);
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = CL;
@@ -2011,7 +2044,7 @@ template <int E, bool FULL, int CL>
 static cudaError_t vocab_seq_tfc(const Dims& D, const Batch& b, const VocabIO& io, int m, const float* zrows,
                                  const int32_t* nb_step, const int32_t* obs_step, const NgSnap* snap,
                                  cudaStream_t s) {
-  const size_t smem = (size_t)step_threads<CL>() * E * sizeof(float);
+  const size_t smem = 2 * (size_t)step_threads<CL>() * E * sizeof(float);
   if (m > kSeqMax) return cudaErrorInvalidValue;
   return launch_kernel_cluster(&k_vocab_seq<E, FULL, CL>, dim3(b.Bmax * CL), dim3(step_threads<CL>()), smem, s,
                                D.pdl, CL, D, b, io, m, b.Bmax, zrows, nb_step, obs_step, snap);
