@@ -54,11 +54,13 @@ struct TcMat {
   CUtensorMap a_dec, b_dec;          // a decode step's maps: 2D, boxes of 32 rows
   int dec_pro = -1;                  // how its operand is made there (DecPro), -1: not used
   CUtensorMap b[2][4];               // per forward buffer set
+  CUtensorMap a2, b2[2][2];          // 2D maps for the tiles of two CTAs per SM (bn 64, 128)
   int M = 0, K = 0;
   int kp = 1;                        // 2: 3D maps, two K blocks per pipeline stage (TcGemm::kp)
-  int bn_dec = 0, bn_pf[kPfBuckets] = {};
+  int bn_dec = 0, bn_pf[kPfBuckets] = {};   // tile code: bn, + kOcc2 for two CTAs per SM
   const float* scale = nullptr;
 };
+constexpr int kOcc2 = 1024;
 static int bn_index(int bn) { return bn == 32 ? 0 : bn == 64 ? 1 : bn == 128 ? 2 : 3; }
 
 // The weights' map (box of 128 rows) and its stage shape: BF16 with K a
@@ -388,10 +390,12 @@ extern "C" void nc_ctx_destroy(nc_ctx* ctx) {
   delete ctx;
 }
 
+// Tile codes worth timing for Bmax rows.
 static int tc_bn_candidates(int Bmax, int* out) {
   int n = 0;
   for (int bn : {32, 64, 128, 256}) {
     out[n++] = bn;
+    if (bn >= 64 && bn <= 128 && Bmax > 128) out[n++] = bn + kOcc2;
     if (bn >= Bmax) break;
   }
   return n;
@@ -467,7 +471,7 @@ static int tc_setup(nc_ctx* ctx) {
     t.M = m.rows;
     t.K = m.cols;
     t.scale = m.scale;
-    if (!tc_encode_weights(t, m.w, esz)) return false;
+    if (!tc_encode_weights(t, m.w, esz) || !tc_encode_tmap(&t.a2, m.w, esz, t.K, t.M, 128)) return false;
     ctx->tc.push_back(t);
     return true;
   };
@@ -489,7 +493,7 @@ static int tc_setup(nc_ctx* ctx) {
   const int probe_idx[5] = {0, 1, 2, 3, (int)ctx->tc.size() - 1};
   const int probe_epi[5] = {EPI_STORE, EPI_RESID, EPI_SWIGLU, EPI_RESID, EPI_LOGITS};
   auto tune = [&](int rows, int* chosen) -> int {
-    int cands[4];
+    int cands[6];
     const int nc = tc_bn_candidates(rows, cands);
     NC_TRY(cudaMemcpy(nB, &rows, 4, cudaMemcpyHostToDevice));
     for (int q = 0; q < 5; ++q) {
@@ -498,16 +502,20 @@ static int tc_setup(nc_ctx* ctx) {
       chosen[q] = cands[0];
       for (int ci = 0; ci < nc; ++ci) {
         TcMat tt = t;
-        if (!tc_encode_operand(tt, &tt.b[0][0], ctx->opnd, esz, rows, cands[ci]))
+        const bool two = cands[ci] >= kOcc2;
+        const int bn = cands[ci] % kOcc2;
+        if (!(two ? tc_encode_tmap(&tt.b[0][0], ctx->opnd, esz, t.K, rows, bn)
+                  : tc_encode_operand(tt, &tt.b[0][0], ctx->opnd, esz, rows, bn)))
           return fail(ctx, NC_ECUDA, "tensor map encoding failed");
         TcGemm g{};
-        g.tmap_a = &tt.a;
+        g.tmap_a = two ? &tt.a2 : &tt.a;
         g.tmap_b = &tt.b[0][0];
         g.M = t.M;
         g.K = t.K;
         g.Bmax = rows;
-        g.bn = cands[ci];
-        g.kp = tt.kp;
+        g.bn = bn;
+        g.kp = two ? 1 : tt.kp;
+        g.occ = two ? 2 : 1;
         g.kind_bf16 = kb;
         g.nB = nB;
         g.w_scale = t.scale;
@@ -567,10 +575,16 @@ static int tc_setup(nc_ctx* ctx) {
           return fail(ctx, NC_ECUDA, "tensor map encoding failed");
       }
     }
+    for (int bi = 0; bi < 2; ++bi)
+      if (!tc_encode_tmap(&t.b2[0][bi], src, esz, t.K, R, 64 << bi))
+        return fail(ctx, NC_ECUDA, "tensor map encoding failed");
     if (ctx->n_fs == 2) {
       const void* src1 = (kb && q == 3) ? ctx->fs[1].opnd2 : ctx->fs[1].opnd;
       for (int bi = 0; bi < 4; ++bi)
         if (!tc_encode_operand(t, &t.b[1][bi], src1, esz, ctx->P, 32 << bi))
+          return fail(ctx, NC_ECUDA, "tensor map encoding failed");
+      for (int bi = 0; bi < 2; ++bi)
+        if (!tc_encode_tmap(&t.b2[1][bi], src1, esz, t.K, ctx->P, 64 << bi))
           return fail(ctx, NC_ECUDA, "tensor map encoding failed");
     }
   }
@@ -1043,14 +1057,17 @@ static cudaError_t launch_model_tc(nc_ctx* ctx, const Batch& b, StepMarks& m, in
       while (k + 1 < kPfBuckets && (ctx->P >> (k + 1)) >= b.Bmax) ++k;
       bn = t.bn_pf[k];
     }
+    const bool two = bn >= kOcc2;
+    bn %= kOcc2;
     TcGemm g{};
-    g.tmap_a = &t.a;
-    g.tmap_b = &t.b[set][bn_index(bn)];
+    g.tmap_a = two ? &t.a2 : &t.a;
+    g.tmap_b = two ? &t.b2[set][bn == 128] : &t.b[set][bn_index(bn)];
     g.M = t.M;
     g.K = t.K;
     g.Bmax = b.Bmax;
     g.bn = bn;
-    g.kp = t.kp;
+    g.kp = two ? 1 : t.kp;
+    g.occ = two ? 2 : 1;
     g.zrows = b.z_out;
     g.kind_bf16 = kb;
     g.nB = b.nB;
@@ -1515,6 +1532,7 @@ static int encode_prefill(nc_ctx* ctx, int n, int m0, const int32_t* tok_dev, co
       fork(s, vs, ctx->ev_fork);
       Dims Dv = D;
       Dv.pdl = 0;                                   // the vocabulary passes: see below
+      int64_t pos = 0;                              // positions of the chunks before
       for (size_t c = 0; c < plan.size() && e == cudaSuccess; ++c) {
         const int mc = plan[c].first, ne = plan[c].second, set = (int)(c & 1), cs = (int)(c % kCodeSets);
         cudaStream_t sc = fst[set];
@@ -1544,6 +1562,7 @@ static int encode_prefill(nc_ctx* ctx, int n, int m0, const int32_t* tok_dev, co
         f.tok = F.f_tok;
         f.z_out = ctx->zrows[cs];
         f.pm = mc;
+        f.len_max = pos += mc;
         LayerSync sync;
         sync.wait = c >= 1 ? ctx->ev_layer[set ^ 1].data() : nullptr;
         sync.rec = ctx->ev_layer[set].data();

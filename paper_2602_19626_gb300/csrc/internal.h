@@ -134,8 +134,8 @@ struct Batch {
   // wait on the previous kernel.
   const float* z_in;
   const int32_t* z_idx;
-  // Decode rows: a bound of the lengths of their streams (0: none known).
-  // The attention's cluster holds the chunks of the longest window.
+  // A bound of the rows' positions + 1 (0: none known): the attention launches
+  // the chunks of the longest window it allows.
   int64_t len_max;
 };
 
@@ -319,6 +319,7 @@ struct TcGemm {
   int M, K, Bmax, bn, kind_bf16;
   int kp;                   // 2: both maps 3D ([K blocks][rows][128 B], tc_encode_tmap3), two K blocks
                             // per stage (BF16, K a multiple of 64); otherwise 2D maps, one per stage
+  int occ;                  // 2: the variant of two CTAs per SM (2D maps, bn 64 or 128)
   const int32_t* nB;        // active rows (device scalar), or nullptr: Bmax
   const float* w_scale;     // FP8: [M]
   const float* x_scale;     // FP8: [Bmax]

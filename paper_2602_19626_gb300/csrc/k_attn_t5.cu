@@ -196,11 +196,22 @@ __global__ void __launch_bounds__(kT5Threads, 2) k_attn_t5(Dims D, Batch b, int 
   StreamDev& st = b.st[slot];
   if (tid < T.nr) a_row[tid] = b.pos[T.row0 + tid];
   __syncthreads();
-  int a_max = -1;
-  for (int r = 0; r < T.nr; ++r) a_max = max(a_max, a_row[r]);
+  // the rows' positions rise up to their stream's end
+  int a_max = a_row[T.nr - 1];
+  for (int r = 0; a_max < 0 && r < T.nr; ++r) a_max = a_row[T.nr - 1 - r];
   const int start = a_max < 0 ? 0 : window_start_at(D, a_max);
   const int nch = a_max < 0 ? 0 : (a_max - start) / kT5Chunk + 1;
-  if (rank >= nch) return;                         // the merge kernel zeroes the rows of no window
+  if (rank >= nch) {
+    // a tile of no window (every row past its stream's end): zeros, by rank 0
+    if (nch == 0 && rank == 0 && p < T.npairs) {
+      pdl_wait();
+      const int rr = (T.pb + p) / grp, hh = (T.pb + p) % grp;
+      for (int i = 0; i < 8; ++i)
+        store_out(io, (size_t)(T.row0 + rr) * D.hq * kHeadDim + (g * grp + hh) * kHeadDim + 32 * wg + 4 * i,
+                  make_float4(0.f, 0.f, 0.f, 0.f));
+    }
+    return;
+  }
   const int c_lo = start + rank * kT5Chunk;
   const int nblk = min(kT5Blocks, (a_max - c_lo) / kT5Block + 1);
   // this thread's pair and its row's position (-1: padding or past the stream's end)
@@ -317,15 +328,29 @@ __global__ void __launch_bounds__(kT5Threads, 2) k_attn_t5(Dims D, Batch b, int 
     ok = __syncthreads_and(ok && mbar_wait(nblk > 2 ? bar_o1 : bar_o0, 0));
     fence_after_sync();
     const float Lc = __fadd_rn(red[p], red[kT5Pairs + p]);
-    // the chunk's (O_c, M_c, l_c) of the present pairs: warpgroup h writes
-    // dims 32 h .. 32 h + 31
-    const int tp = min(kT5Pairs, b.pm * grp);   // pairs a tile can hold
+    // the chunk's (O_c, M_c, l_c) of the present pairs: warpgroup h takes
+    // dims 32 h .. 32 h + 31.  A tile of one chunk is merged here (merge_chunks
+    // of one chunk, whose factor is exp(0) = 1); else they go to the partials.
+    const int tp = min(kT5Pairs, b.pm * grp);      // pairs a tile can hold
     float4* part = part_base(D, (size_t)blockIdx.z * D.hkv + g, tp);
     if (ok && mine) {
       uint32_t r[32];
       tmem_ld32_nowait(tlane + 32 * wg, r);
       tmem_wait_ld();
-      if (p < T.npairs && my_a >= c_lo) {
+      if (nch == 1) {
+        if (p < T.npairs) {
+          const size_t off = (size_t)(T.row0 + my_r) * D.hq * kHeadDim + (g * grp + my_h) * kHeadDim + 32 * wg;
+          const float l = my_a >= 0 ? __fmaf_rn(Lc, 1.f, 0.f) : 1.f;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            float o[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              o[q] = my_a >= 0 ? __fdiv_rn(__fmaf_rn(__uint_as_float(r[4 * i + q]), 1.f, 0.f), l) : 0.f;
+            store_out(io, off + 4 * i, make_float4(o[0], o[1], o[2], o[3]));
+          }
+        }
+      } else if (p < T.npairs && my_a >= c_lo) {
 #pragma unroll
         for (int i = 0; i < 8; ++i)
           __stcg(part + (size_t)(rank * kGroups + 8 * wg + i) * tp + p,
@@ -360,9 +385,15 @@ __global__ void __launch_bounds__(kT5Threads) k_attn_merge(Dims D, Batch b, int 
   const T5Tile T = t5_tile(b, grp, tps, blockIdx.x);
   const int p = blockIdx.z * kMergePairs + (threadIdx.x % kMergePairs), i = threadIdx.x / kMergePairs;
   if (T.row0 >= *b.nB) return;
+  // the positions were written several launches back; a tile of one chunk was
+  // merged, and one of none (all rows past their streams' ends) zeroed, by
+  // its attention CTA
+  int a_max = b.pos[T.row0 + T.nr - 1];
+  for (int r = 1; a_max < 0 && r < T.nr; ++r) a_max = b.pos[T.row0 + T.nr - 1 - r];
+  const bool one = a_max < 0 || (a_max - window_start_at(D, a_max)) / kT5Chunk == 0;
   pdl_wait();
   pdl_trigger();
-  if (p >= T.npairs) return;
+  if (one || p >= T.npairs) return;
   const int my_r = (T.pb + p) / grp, my_h = (T.pb + p) % grp;
   const int a = b.pos[T.row0 + my_r];
   const int ncp = a < 0 ? 0 : (a - window_start_at(D, a)) / kT5Chunk + 1;
@@ -373,12 +404,17 @@ __global__ void __launch_bounds__(kT5Threads) k_attn_merge(Dims D, Batch b, int 
 }
 
 // Prefill append: row j's k (rotated at its position a) and v, rounded to
-// BF16, into the ring of `layer`, and its grp query heads of KV head g,
-// rotated, scaled by 1/8 and rounded to BF16, into q16 (the attention's
-// decode step does the same arithmetic for its one row).
-__global__ void __launch_bounds__(128) k_kv_append_t5(Dims D, Batch b, int layer, const float* qkv) {
-  const int j = blockIdx.y, g = blockIdx.x, tid = threadIdx.x;
-  const int grp = D.hq / D.hkv;
+// BF16, into the ring of `layer`, and its query heads, rotated, scaled by 1/8
+// and rounded to BF16, into q16 (the attention's decode step does the same
+// arithmetic for its one row).  Sixteen threads take a row, thread i the
+// rotation pairs 2 i and 2 i + 1 of every head, so a position's rotations are
+// formed once and all heads' loads are in flight together (a CTA per row and
+// KV head took 13.8 us for 3,072 rows, most of it waiting).
+constexpr int kAppendThreads = 128, kAppendRows = kAppendThreads / 16;
+template <int HQ, int HKV>
+__global__ void __launch_bounds__(kAppendThreads) k_kv_append_t5(Dims D, Batch b, int layer, const float* qkv) {
+  const int hq = HQ ? HQ : D.hq, hkv = HKV ? HKV : D.hkv;
+  const int j = blockIdx.x * kAppendRows + (threadIdx.x >> 4), dd = 2 * (threadIdx.x & 15);
   pdl_wait();
   pdl_trigger();
   if (j >= *b.nB) return;
@@ -386,29 +422,33 @@ __global__ void __launch_bounds__(128) k_kv_append_t5(Dims D, Batch b, int layer
   if (a < 0) return;
   StreamDev& st = b.st[b.slots[j]];
   const float* row = qkv + (size_t)j * D.qkv_rows;
-  const size_t ri = (size_t)(a & (D.L - 1)) * kHeadDim;
-  __nv_bfloat16* kv = static_cast<__nv_bfloat16*>(st.kv);
-  __nv_bfloat16* q16 = static_cast<__nv_bfloat16*>(D.q16) + (size_t)j * D.hq * kHeadDim;
-  for (int e = tid; e < (grp + 1) * (kHeadDim / 2); e += blockDim.x) {
-    const int h = e / (kHeadDim / 2), dd = e % (kHeadDim / 2);
-    const float2 c = rope_cs(D, a, dd);
-    if (h < grp) {
-      const float* src = row + (g * grp + h) * kHeadDim;
-      const float2 rr = rope_rotate(__ldcg(src + dd), __ldcg(src + dd + kHeadDim / 2), c);
-      __nv_bfloat16* dst = q16 + (g * grp + h) * kHeadDim;
-      dst[dd] = __float2bfloat16_rn(rr.x * 0.125f);
-      dst[dd + kHeadDim / 2] = __float2bfloat16_rn(rr.y * 0.125f);
+  __nv_bfloat16* ring = static_cast<__nv_bfloat16*>(st.kv) + attn_plane_off(D, layer, 0) +
+                        (size_t)(a & (D.L - 1)) * kHeadDim;
+  const size_t plane = (size_t)D.L * kHeadDim;
+  __nv_bfloat16* q16 = static_cast<__nv_bfloat16*>(D.q16) + (size_t)j * hq * kHeadDim;
+  const float2 c0 = rope_cs(D, a, dd), c1 = rope_cs(D, a, dd + 1);
+  auto put = [](__nv_bfloat16* dst, float x, float y) { *reinterpret_cast<uint32_t*>(dst) = pack_bf16(x, y); };
+#pragma unroll
+  for (int h = 0; h < hq + hkv; ++h) {             // the query heads, then the keys
+    const float* src = row + h * kHeadDim + dd;
+    const float2 x = __ldcg(reinterpret_cast<const float2*>(src));
+    const float2 y = __ldcg(reinterpret_cast<const float2*>(src + kHeadDim / 2));
+    const float2 r0 = rope_rotate(x.x, y.x, c0), r1 = rope_rotate(x.y, y.y, c1);
+    if (h < hq) {
+      put(q16 + h * kHeadDim + dd, r0.x * 0.125f, r1.x * 0.125f);
+      put(q16 + h * kHeadDim + dd + kHeadDim / 2, r0.y * 0.125f, r1.y * 0.125f);
     } else {
-      const float* src = row + D.hq * kHeadDim + g * kHeadDim;
-      const float2 rr = rope_rotate(__ldcg(src + dd), __ldcg(src + dd + kHeadDim / 2), c);
-      __nv_bfloat16* dst = kv + attn_plane_off(D, layer, g) + ri;
-      dst[dd] = __float2bfloat16_rn(rr.x);
-      dst[dd + kHeadDim / 2] = __float2bfloat16_rn(rr.y);
+      __nv_bfloat16* dst = ring + (size_t)(h - hq) * plane + dd;
+      put(dst, r0.x, r1.x);
+      put(dst + kHeadDim / 2, r0.y, r1.y);
     }
   }
-  if (tid < kHeadDim)
-    kv[attn_plane_off(D, layer, D.hkv + g) + ri + tid] =
-        __float2bfloat16_rn(__ldcg(row + (D.hq + D.hkv) * kHeadDim + g * kHeadDim + tid));
+#pragma unroll
+  for (int h = 0; h < hkv; ++h) {
+    const float4 v = __ldcg(reinterpret_cast<const float4*>(row + (hq + hkv + h) * kHeadDim + 2 * dd));
+    *reinterpret_cast<uint2*>(ring + (size_t)(hkv + h) * plane + 2 * dd) =
+        make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+  }
 }
 
 }  // namespace
@@ -438,9 +478,14 @@ cudaError_t launch_attn_t5(const Dims& D, const Batch& b, int layer, const float
   const size_t tp = std::min(kT5Pairs, b.pm * grp);
   if ((size_t)tiles * D.hkv * kT5MaxRanks * tp * kPartRow > D.attn_part_cap) return cudaErrorInvalidValue;
   const AttnIO io{qkv, attn_out, out16};
-  cudaError_t e = launch_kernel(k_attn_t5, dim3(kT5MaxRanks, D.hkv, tiles), dim3(kT5Threads), kT5Smem, s, D.pdl, D, b,
+  // chunks of the longest window of the launch: a CTA without a chunk costs
+  // its launch and three dependent loads, more than a third of the kernel
+  // when all eight were launched for windows of one
+  const int64_t len = b.len_max > 0 && b.len_max < D.L ? b.len_max : D.L;
+  const int nch = (int)((len + kT5Chunk - 1) / kT5Chunk);
+  cudaError_t e = launch_kernel(k_attn_t5, dim3(nch, D.hkv, tiles), dim3(kT5Threads), kT5Smem, s, D.pdl, D, b,
                                 layer, tps, io);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && nch > 1)
     e = launch_kernel(k_attn_merge, dim3(tiles, D.hkv, kT5Pairs / kMergePairs), dim3(kT5Threads), 0, s, D.pdl, D, b,
                       tps, io);
   return e;
@@ -448,7 +493,10 @@ cudaError_t launch_attn_t5(const Dims& D, const Batch& b, int layer, const float
 
 cudaError_t launch_kv_append_t5(const Dims& D, const Batch& b, int layer, const float* qkv, cudaStream_t s) {
   if (!D.q16) return cudaErrorInvalidValue;
-  return launch_kernel(k_kv_append_t5, dim3(D.hkv, b.Bmax), dim3(128), 0, s, D.pdl, D, b, layer, qkv);
+  const dim3 grid((b.Bmax + kAppendRows - 1) / kAppendRows);
+  if (D.hq == 9 && D.hkv == 3)                     // the full model's heads: the loops unrolled
+    return launch_kernel(k_kv_append_t5<9, 3>, grid, dim3(kAppendThreads), 0, s, D.pdl, D, b, layer, qkv);
+  return launch_kernel(k_kv_append_t5<0, 0>, grid, dim3(kAppendThreads), 0, s, D.pdl, D, b, layer, qkv);
 }
 
 }  // namespace nc

@@ -191,15 +191,7 @@ __global__ void __launch_bounds__(NW * 32, 1)
         for (int i = 0; i < kPlainVecs; ++i) {
           const int c = 4 * (lane + 32 * i);
           if (c < nk * kPer) {
-            uint32_t w = 0;
-            if (c < g.K) {
-              const float f[4] = {v[q][i].x, v[q][i].y, v[q][i].z, v[q][i].w};
-#pragma unroll
-              for (int e = 0; e < 4; e += 2)
-                w |= (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(__fdiv_rn(f[e], s), __fdiv_rn(f[e + 1], s)),
-                                                        __NV_SATFINITE, __NV_E4M3)
-                     << (8 * e);
-            }
+            const uint32_t w = c < g.K ? fp8x4(v[q][i], s) : 0u;
             *reinterpret_cast<uint32_t*>(sB + op_off<1, BN>(j, c)) = w;
           }
         }

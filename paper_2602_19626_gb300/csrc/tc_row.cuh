@@ -79,4 +79,11 @@ __device__ __forceinline__ float fp8_scale(float m) {
   return m > 0.f ? __fdiv_rn(m, 448.0f) : 1.0f;
 }
 
+// Four values over the scale s as E4M3 bytes.
+__device__ __forceinline__ uint32_t fp8x4(const float4& v, float s) {
+  const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(__fdiv_rn(v.x, s), __fdiv_rn(v.y, s)), __NV_SATFINITE, __NV_E4M3);
+  const uint32_t hi = __nv_cvt_float2_to_fp8x2(make_float2(__fdiv_rn(v.z, s), __fdiv_rn(v.w, s)), __NV_SATFINITE, __NV_E4M3);
+  return lo | (hi << 16);
+}
+
 }  // namespace nc
