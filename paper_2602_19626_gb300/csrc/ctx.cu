@@ -826,8 +826,9 @@ static int slot_alloc(nc_ctx* ctx, Slot& s, int64_t max_len) {
       if (!tc_encode_tmap(&map, s.kv, 2, kHeadDim, (int64_t)D.n_layers * 2 * D.hkv * D.L, 64))
         return fail(ctx, NC_ECUDA, "KV tensor map encoding failed");
       const int si = (int)(&s - ctx->slots.data());
-      NC_TRY(cudaMemcpy(static_cast<unsigned char*>(const_cast<void*>(D.kv_tmap)) + (size_t)si * kTmapBytes, &map,
-                        kTmapBytes, cudaMemcpyHostToDevice));
+      NC_TRY(cudaMemcpyAsync(static_cast<unsigned char*>(const_cast<void*>(D.kv_tmap)) + (size_t)si * kTmapBytes, &map,
+                             kTmapBytes, cudaMemcpyHostToDevice, ctx->stream));
+      NC_TRY(cudaStreamSynchronize(ctx->stream));   // the map is this frame's (once per slot)
     }
     s.kv_ready = true;
   }

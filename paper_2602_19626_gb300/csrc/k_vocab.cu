@@ -244,11 +244,18 @@ __device__ __forceinline__ uint4 as_u4(const T& v) {
   static_assert(sizeof(T) == 16, "16-byte values");
   return *reinterpret_cast<const uint4*>(&v);
 }
-// Lanes 0 .. CL - 1: the warp's partial v to its global index in the array
-// `mine` of CTA `lane`.
+// Lanes 0 .. CL - 1: the warp's partial v to its entry in the array `mine` of
+// CTA `lane`.  Global warp gw sits at 32 (gw mod 4) + gw / 4, so that lane l
+// reads the four of warps 4 l .. 4 l + 3 at l, l + 32, .. without bank conflicts.
 template <int CL, typename T>
 __device__ __forceinline__ void push_part_async(T* mine, const Lanes& L, T v, uint64_t* bar) {
-  if (L.lane < CL) st_async16(remote_addr(smem_addr(mine + L.gw), L.lane), remote_addr(smem_addr(bar), L.lane), as_u4(v));
+  const int at = 32 * (L.gw & 3) + (L.gw >> 2);
+  if (L.lane < CL) st_async16(remote_addr(smem_addr(mine + at), L.lane), remote_addr(smem_addr(bar), L.lane), as_u4(v));
+}
+template <typename T>
+__device__ __forceinline__ void async_parts(const T* arr, int lane, T (&v)[4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = arr[32 * i + lane];
 }
 __device__ __forceinline__ void xbar_arm(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
@@ -289,21 +296,33 @@ __device__ __forceinline__ void local_parts(const T* arr, int lane, T (&v)[4]) {
 // in the order k = 0, 1, 2); each lane then reads its E sums and zeroes them.
 template <int E>
 __device__ __forceinline__ void ngram_scatter(const NgSnap& g, float* spw, const Lanes& L) {
-  constexpr int kSpan = 32 * E;
-  __syncwarp();                                    // the region's last reads and zeroes are done
+  constexpr int kSpan = 32 * E, kPer = kMaxSlots / 32;
+  // all slots first: few of them, if any, lie in the warp's symbols
+  int at[kMaxOrder][kPer];
+  float mass[kMaxOrder][kPer];
+  bool any = false;
 #pragma unroll
   for (int k = 0; k < kMaxOrder; ++k) {
     const int ns = g.ns[k];
     const float coef = g.coef[k];
 #pragma unroll
-    for (int h = 0; h < kMaxSlots / 32; ++h) {
+    for (int h = 0; h < kPer; ++h) {
       const int q = L.lane + 32 * h;
-      if (q < ns) {
-        const int2 tc = g.tc[k][q];
-        const int t = tc.x - L.wbase;
-        if ((unsigned)t < (unsigned)kSpan) spw[t] = __fadd_rn(spw[t], __fmul_rn(coef, (float)tc.y));
-      }
+      const int2 tc = g.tc[k][q];                  // past the entry's slots: stale, not used
+      const int t = tc.x - L.wbase;
+      const bool in = q < ns && (unsigned)t < (unsigned)kSpan;
+      at[k][h] = in ? t : -1;
+      mass[k][h] = __fmul_rn(coef, (float)tc.y);
+      any |= in;
     }
+  }
+  if (!__any_sync(0xffffffffu, any)) return;
+  __syncwarp();                                    // the region's last reads and zeroes are done
+#pragma unroll
+  for (int k = 0; k < kMaxOrder; ++k) {
+#pragma unroll
+    for (int h = 0; h < kPer; ++h)
+      if (at[k][h] >= 0) spw[at[k][h]] = __fadd_rn(spw[at[k][h]], mass[k][h]);
     __syncwarp();
   }
 }
@@ -512,6 +531,7 @@ __device__ __forceinline__ uint4 quant_part(const float (&p)[E], const Lanes& L,
 struct Quant {
   long long resid, woff;
   int argmax;
+  uint32_t maxv;             // the first maximum's value bits
   bool bad;
 };
 __device__ __forceinline__ Quant quant_reduce(const uint4 (&v)[4], const Lanes& L, uint32_t T) {
@@ -535,8 +555,19 @@ __device__ __forceinline__ Quant quant_reduce(const uint4 (&v)[4], const Lanes& 
   q.resid = (long long)T - (long long)tot;
   q.woff = (long long)off;
   q.argmax = (int)ix;
+  q.maxv = hi;
   q.bad = __any_sync(0xffffffffu, bad);
   return q;
+}
+
+// The exponential-weights step of the mixer (Sec. 3.5) with the observed
+// token's log p_tilde and p_ng.
+__device__ __forceinline__ void log_loss_step(const Dims& D, float pngs, float lpt, float& th0, float& th1) {
+  const float a0 = __fmaf_rn(D.eta, lpt, th0), a1 = __fmaf_rn(D.eta, __logf(pngs), th1);
+  const float am = fmaxf(a0, a1);
+  const float lse = __fadd_rn(am, __logf(__fadd_rn(exp_fast(__fsub_rn(a0, am)), exp_fast(__fsub_rn(a1, am)))));
+  th0 = __fsub_rn(a0, lse);
+  th1 = __fsub_rn(a1, lse);
 }
 
 // Mixer update with the observed token (Sec. 3.5): exponential weights with
@@ -553,11 +584,7 @@ __device__ __forceinline__ void mixer_update(const Dims& D, bool mixing, float2 
     th0 = __fsub_rn(th0, __fmul_rn(D.alpha, __fsub_rn(w.x, r0)));
     th1 = __fsub_rn(th1, __fmul_rn(D.alpha, __fsub_rn(w.y, r1)));
   } else {
-    const float a0 = __fmaf_rn(D.eta, lpt, th0), a1 = __fmaf_rn(D.eta, __logf(pngs), th1);
-    const float am = fmaxf(a0, a1);
-    const float lse = __fadd_rn(am, __logf(__fadd_rn(exp_fast(__fsub_rn(a0, am)), exp_fast(__fsub_rn(a1, am)))));
-    th0 = __fsub_rn(a0, lse);
-    th1 = __fsub_rn(a1, lse);
+    log_loss_step(D, pngs, lpt, th0, th1);
   }
 }
 
@@ -807,7 +834,9 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1) k_vocab(Dims D, Batch b
 // the earliest, after every warp's round k + 2.
 //
 // Measured (GB300, one stream of 8,192 tokens, 16 CTAs): 3.1 us a position when
-// coding a position came before the next one's partials, 2.4 us now.
+// coding a position came before the next one's partials, 1.9 us now (3,850 cycles: 840
+// scores and partials, 1,850 in the window, which hides the round's travel, 340
+// left to wait, 830 reduction and head step).
 constexpr int kSeqSlots = 4;
 constexpr uint32_t kRoundPart = kClusterWarps * 16;        // bytes of one array of warp partials
 struct SeqShared {
@@ -818,6 +847,7 @@ struct SeqShared {
   } slot[kSeqSlots];
   NgSnap ng[kSnapBufs];         // N-gram states of the positions ahead
   uint64_t xbar[kSeqSlots];     // the rounds' barriers
+  uint2 pend[kSeqSlots];        // the coded token's counts below it in its warp, and its own, until it is finished
   int32_t obs[kSeqMax], nb[kSeqMax];   // the chunk's tokens and active rows, per position
 };
 
@@ -901,34 +931,39 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1)
     return h;
   };
 
-  // coded positions not yet finished: [0] the last one coded, [1], [2] before it
-  struct Pend {
-    int t, pos, am_i;
-    uint32_t below, ct, am_c;
-    bool own;
-  } pend[3];
   // the position before the current one, not yet coded
   float pt[E];
   Soft sm{0.f, 0.f, 0.f};
   float2 w = mix_weights(th0, th1);              // the weights of the position to be coded next
   float cu = 0.f, cu_next = 0.f, h = 0.f;
-  int t_prev = -1;
   bool skipped = false, mixing = false;
   bool xok = true;                               // no exchange wait has given up
   int r = 0;
 
-  // the observed token's p_tilde, p_ng and log p_tilde at the position whose
-  // exchange is (o, sm): the owner's arithmetic
-  auto obs_step_mixer = [&](const float4& o, float& scale) {
+  // the observed token's p_tilde at the position whose exchange is (o, sm):
+  // the owner's arithmetic
+  auto obs_prob = [&](const float4& o) {
     const float f = o.y == -INFINITY ? 0.f : __fdividef(exp_fast(__fsub_rn(o.y, sm.M)), sm.S);
-    const float pts = __fmul_rn(o.x, f);
-    mixer_update(D, mixing, w, pts, o.w, __fsub_rn(__fsub_rn(o.z, sm.M), __logf(sm.S)), th0, th1, scale);
-    last_pts = pts;
-    last_pngs = o.w;
+    return __fmul_rn(o.x, f);
   };
   // code position q = r - 1: the mix, its counts and their partials into the
   // slot of round q + 2; then its mixer step and counts
   auto code = [&](int q) {
+    const int tq = sh.obs[q];
+    // the log-loss mixer's step first, without a branch: a chain of scalar
+    // functions to run beside the rest
+    if (!nll) {
+      const float4 o = sh.slot[q & 3].obs;
+      const float pts = obs_prob(o), lpt = __fsub_rn(__fsub_rn(o.z, sm.M), __logf(sm.S));
+      float t0 = th0, t1 = th1;
+      log_loss_step(D, o.w, lpt, t0, t1);
+      const bool step = mixing && !skipped;
+      th0 = step ? t0 : th0;
+      th1 = step ? t1 : th1;
+      last_pts = skipped ? last_pts : pts;
+      last_pngs = skipped ? last_pngs : o.w;
+    }
+    const float2 w_next = mix_weights(th0, th1);
     const size_t prow = (size_t)(io.probe_row ? io.probe_row[j] : j) * V;
     const bool probe = io.probe_tok == (int64_t)(n0 + q + 1);
     float png[E];
@@ -940,45 +975,49 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1)
     }
     if (probe && io.probe_png) store_run<E>(io.probe_png + prow, L.v0, V, png);
     float p[E];
-    coded_probs<E>(pt, png, w, skipped, mixing, p);
+    if (D.skip) {
+      coded_probs<E>(pt, png, w, skipped, mixing, p);
+    } else {                                     // without mixing, the weights (1, 0) give p_tilde itself
+      const float w0 = mixing ? w.x : 1.f, w1 = mixing ? w.y : 0.f;
+#pragma unroll
+      for (int i = 0; i < E; ++i) p[i] = __fmaf_rn(w0, pt[i], __fmul_rn(w1, png[i]));
+    }
     if (probe && io.probe_p) store_run<E>(io.probe_p + prow, L.v0, V, p);
     uint32_t c[E], excl = 0;
-    const bool here = t_prev >= L.wbase && t_prev < L.wbase + 32 * E;
-    const bool owner = t_prev >= L.v0 && t_prev < L.v0 + E;
-    pend[2] = pend[1];
-    pend[1] = pend[0];
-    Pend& n = pend[0];
-    const uint4 qp = quant_part<E, FULL>(p, L, V, K, Kf, D.floor, io.intervals && here, finite_step(sm, w), c, excl,
-                                         n.am_i, n.am_c);
+    const bool here = tq >= L.wbase && tq < L.wbase + 32 * E;
+    const bool owner = tq >= L.v0 && tq < L.v0 + E;
+    int am_i;
+    uint32_t am_c;
+    const uint4 qp = quant_part<E, FULL>(p, L, V, K, Kf, D.floor, here, finite_step(sm, w), c, excl,
+                                         am_i, am_c);
     push_part_async<CL>(sh.slot[(q + 2) & 3].qn, L, qp, &sh.xbar[(q + 2) & 3]);
-    n.own = owner && io.intervals;
-    n.t = t_prev;
-    n.pos = n0 + q;
     if (owner) {
-      counts_around<E>(c, L.v0, t_prev, n.below, n.ct);
-      n.below += excl;
+      uint32_t below, ct;
+      counts_around<E>(c, L.v0, tq, below, ct);
+      sh.pend[q & 3] = make_uint2(below + excl, ct);
       if (ngram) {
 #pragma unroll
         for (int i = 0; i < E; ++i)
-          if (L.v0 + i == t_prev) cnt[i] += 1;
+          if (L.v0 + i == tq) cnt[i] += 1;
       }
     }
-    if (!nll && !skipped) {
-      float scale;
-      obs_step_mixer(sh.slot[q & 3].obs, scale);
-    }
-    w = mix_weights(th0, th1);
+    w = w_next;
   };
-  // interval and numeric checks of position q, pending as `n`, from the
-  // partials that came with round q + 2
-  auto finish = [&](int q, const Pend& n) {
+  // interval and numeric checks of position q from the partials that came
+  // with round q + 2
+  auto finish = [&](int q) {
+    const int tq = sh.obs[q];
+    if (tq < L.wbase || tq >= L.wbase + 32 * E) return;   // the token's warp
     uint4 qv[4];
-    local_parts(sh.slot[(q + 2) & 3].qn, L.lane, qv);
+    async_parts(sh.slot[(q + 2) & 3].qn, L.lane, qv);
     const Quant qr = quant_reduce(qv, L, T);
-    if (n.own)
-      write_interval(io.intervals + 2 * ((size_t)j * io.interval_stride + n.pos), qr, n.t, n.below, n.ct);
-    if ((qr.bad && L.rank == 0 && threadIdx.x == 0) || final_count_bad(qr, n.am_i, n.am_c, D.floor, T))
-      atomicOr(&st.status, ST_NUMERIC);
+    if (tq >= L.v0 && tq < L.v0 + E) {           // the thread that coded it
+      const uint2 n = sh.pend[q & 3];
+      write_interval(io.intervals + 2 * ((size_t)j * io.interval_stride + n0 + q), qr, tq, n.x, n.y);
+      bool bad = qr.bad;                         // and the first maximum's final count stays within [floor, T]
+      const long long cf = (long long)max(floor_count(__uint_as_float(qr.maxv), K, Kf, bad), D.floor) + qr.resid;
+      if (bad || cf < (long long)D.floor || cf > (long long)T) atomicOr(&st.status, ST_NUMERIC);
+    }
   };
   auto wait_round = [&](int k) {
     xok = __all_sync(0xffffffffu, xbar_wait(&sh.xbar[k & 3], (uint32_t)(k >> 2) & 1u));
@@ -1012,7 +1051,8 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1)
     if (t >= L.wbase && t < L.wbase + 32 * E) {  // the observed token's warp
       float png_t = 0.f;
       if (ngram && t >= L.v0 && t < L.v0 + E)    // counts up to position r - 2, and r - 1's token
-        png_t = __fmaf_rn(cu_next, (float)(pick<E>(cnt, L.v0, t) + 1 + (t == t_prev ? 1 : 0)), spw(r)[t - L.wbase]);
+        png_t = __fmaf_rn(cu_next, (float)(pick<E>(cnt, L.v0, t) + 1 + (r > 0 && t == sh.obs[r - 1] ? 1 : 0)),
+                          spw(r)[t - L.wbase]);
       const int src = (t - L.wbase) / E;
       const float4 o = make_float4(__shfl_sync(0xffffffffu, pick<E>(e, L.v0, t), src), part.x,
                                    __shfl_sync(0xffffffffu, pick<E>(s, L.v0, t), src),
@@ -1024,7 +1064,7 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1)
     const bool more = r + 1 < R;
     if (more) load_runf<E, FULL>(zj + (size_t)(r + 1) * V, L.v0, V, z, -INFINITY);
     if (r >= 1) code(r - 1);
-    if (r >= 3) finish(r - 3, pend[2]);
+    if (r >= 3) finish(r - 3);
     cu = cu_next;
     if (ngram && more) {
       ngram_scatter<E>(sh.ng[(r + 1) % kSnapBufs], spw(r + 1), L);
@@ -1035,13 +1075,18 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1)
     if (!wait_round(r)) break;                   // the other warps give up on their next round
     // ---- the chain: position r's probabilities and head step
     float4 smv[4];
-    local_parts(in.sm, L.lane, smv);
+    async_parts(in.sm, L.lane, smv);
     sm = softmax_reduce(smv, D.skip != 0);
     skipped = D.skip && sm.H < kSkipBits;
     mixing = ngram && n0 + r + 1 > D.warmup;
     probs_tilde<E>(e, part.x, sm, pt);
     float scale = 1.f;
-    if (nll && !skipped) obs_step_mixer(in.obs, scale);   // the head's step needs the mixer's
+    if (nll && !skipped) {                       // the head's step needs the mixer's
+      const float4 o = in.obs;
+      last_pts = obs_prob(o);
+      last_pngs = o.w;
+      mixer_update(D, mixing, w, last_pts, o.w, 0.f, th0, th1, scale);
+    }
     if (!skipped && D.use_head)
       head_update<E>(bias, pt, __fmul_rn(D.alpha, scale), L.v0, t, t >= L.v0 && t < L.v0 + E);
     if (probe && io.probe_pt) store_run<E>(io.probe_pt + prow, L.v0, V, pt);
@@ -1051,19 +1096,18 @@ __global__ void __launch_bounds__(step_threads<CL>(), 1)
       if (r + kSnapBufs < R) snap_copy_async(&sh.ng[r % kSnapBufs], gj + r + kSnapBufs);
       else cp_async_commit();
     }
-    t_prev = t;
   }
   // ---- the last positions: code r - 1, finish r - 3, r - 2 and r - 1
   if (r > 0 && xok) {
     code(r - 1);
-    if (r >= 3) finish(r - 3, pend[2]);
+    if (r >= 3) finish(r - 3);
     if (r >= 2) {
       if (threadIdx.x == 0) xbar_arm(&sh.xbar[r & 3], kRoundPart);
-      if (wait_round(r)) finish(r - 2, pend[1]);
+      if (wait_round(r)) finish(r - 2);
     }
     if (xok) {
       if (threadIdx.x == 0) xbar_arm(&sh.xbar[(r + 1) & 3], kRoundPart);
-      if (wait_round(r + 1)) finish(r - 1, pend[0]);
+      if (wait_round(r + 1)) finish(r - 1);
     }
   }
   if (!xok && L.lane == 0) atomicOr(&st.status, ST_TIMEOUT);
