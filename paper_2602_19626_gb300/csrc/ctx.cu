@@ -54,7 +54,7 @@ struct TcMat {
   CUtensorMap a_dec, b_dec;          // a decode step's maps: 2D, boxes of 32 rows
   int dec_pro = -1;                  // how its operand is made there (DecPro), -1: not used
   CUtensorMap b[2][4];               // per forward buffer set
-  CUtensorMap a2, b2[2][2];          // 2D maps for the tiles of two CTAs per SM (bn 64, 128)
+  CUtensorMap a2, b2[2][3];          // 2D maps for the tiles of two CTAs per SM (bn 32, 64, 128)
   int M = 0, K = 0;
   int kp = 1;                        // 2: 3D maps, two K blocks per pipeline stage (TcGemm::kp)
   int bn_dec = 0, bn_pf[kPfBuckets] = {};   // tile code: bn, + kOcc2 for two CTAs per SM
@@ -395,7 +395,7 @@ static int tc_bn_candidates(int Bmax, int* out) {
   int n = 0;
   for (int bn : {32, 64, 128, 256}) {
     out[n++] = bn;
-    if (bn >= 64 && bn <= 128 && Bmax > 128) out[n++] = bn + kOcc2;
+    if (bn <= 128) out[n++] = bn + kOcc2;
     if (bn >= Bmax) break;
   }
   return n;
@@ -493,7 +493,7 @@ static int tc_setup(nc_ctx* ctx) {
   const int probe_idx[5] = {0, 1, 2, 3, (int)ctx->tc.size() - 1};
   const int probe_epi[5] = {EPI_STORE, EPI_RESID, EPI_SWIGLU, EPI_RESID, EPI_LOGITS};
   auto tune = [&](int rows, int* chosen) -> int {
-    int cands[6];
+    int cands[7];
     const int nc = tc_bn_candidates(rows, cands);
     NC_TRY(cudaMemcpy(nB, &rows, 4, cudaMemcpyHostToDevice));
     for (int q = 0; q < 5; ++q) {
@@ -525,19 +525,21 @@ static int tc_setup(nc_ctx* ctx) {
         g.h16 = kb ? scratch : nullptr;             // the forward's SwiGLU output format
         g.zrows = scratch;
         g.status = ctx->d_status;
-        // the best of four samples of five back-to-back launches (the first
-        // sample also loads the kernel)
+        // a first launch that also loads the kernel, a second that tells how
+        // long it takes, then the best of three samples of five back-to-back
+        // launches each, or of one where a launch takes over 40 us
         float ms_best = 1e30f;
-        for (int rep = 0; rep < 4; ++rep) {
+        for (int rep = 0, n = 1; rep < 5; ++rep) {
           cudaEventRecord(e0, ctx->stream);
           cudaError_t e = cudaSuccess;
-          for (int k = 0; k < 5 && e == cudaSuccess; ++k) e = launch_gemm_tc(g, probe_epi[q], ctx->stream, false);
+          for (int k = 0; k < n && e == cudaSuccess; ++k) e = launch_gemm_tc(g, probe_epi[q], ctx->stream, false);
           cudaEventRecord(e1, ctx->stream);
           if (e == cudaSuccess) e = cudaEventSynchronize(e1);
           if (e != cudaSuccess) return fail_cuda(ctx, e, "tensor-core autotune");
           float ms = 0.f;
           cudaEventElapsedTime(&ms, e0, e1);
-          if (rep) ms_best = std::min(ms_best, ms);
+          if (rep > 1) ms_best = std::min(ms_best, ms / n);
+          else if (rep == 1) n = ms > 0.04f ? 1 : 5;
         }
         if (ms_best < best) {
           best = ms_best;
@@ -575,16 +577,16 @@ static int tc_setup(nc_ctx* ctx) {
           return fail(ctx, NC_ECUDA, "tensor map encoding failed");
       }
     }
-    for (int bi = 0; bi < 2; ++bi)
-      if (!tc_encode_tmap(&t.b2[0][bi], src, esz, t.K, R, 64 << bi))
+    for (int bi = 0; bi < 3; ++bi)
+      if (!tc_encode_tmap(&t.b2[0][bi], src, esz, t.K, R, 32 << bi))
         return fail(ctx, NC_ECUDA, "tensor map encoding failed");
     if (ctx->n_fs == 2) {
       const void* src1 = (kb && q == 3) ? ctx->fs[1].opnd2 : ctx->fs[1].opnd;
       for (int bi = 0; bi < 4; ++bi)
         if (!tc_encode_operand(t, &t.b[1][bi], src1, esz, ctx->P, 32 << bi))
           return fail(ctx, NC_ECUDA, "tensor map encoding failed");
-      for (int bi = 0; bi < 2; ++bi)
-        if (!tc_encode_tmap(&t.b2[1][bi], src1, esz, t.K, ctx->P, 64 << bi))
+      for (int bi = 0; bi < 3; ++bi)
+        if (!tc_encode_tmap(&t.b2[1][bi], src1, esz, t.K, ctx->P, 32 << bi))
           return fail(ctx, NC_ECUDA, "tensor map encoding failed");
     }
   }
@@ -1062,7 +1064,7 @@ static cudaError_t launch_model_tc(nc_ctx* ctx, const Batch& b, StepMarks& m, in
     bn %= kOcc2;
     TcGemm g{};
     g.tmap_a = two ? &t.a2 : &t.a;
-    g.tmap_b = two ? &t.b2[set][bn == 128] : &t.b[set][bn_index(bn)];
+    g.tmap_b = two ? &t.b2[set][bn_index(bn)] : &t.b[set][bn_index(bn)];
     g.M = t.M;
     g.K = t.K;
     g.Bmax = b.Bmax;

@@ -319,7 +319,7 @@ struct TcGemm {
   int M, K, Bmax, bn, kind_bf16;
   int kp;                   // 2: both maps 3D ([K blocks][rows][128 B], tc_encode_tmap3), two K blocks
                             // per stage (BF16, K a multiple of 64); otherwise 2D maps, one per stage
-  int occ;                  // 2: the variant of two CTAs per SM (2D maps, bn 64 or 128)
+  int occ;                  // 2: the variant of two CTAs per SM (2D maps, bn 32, 64 or 128)
   const int32_t* nB;        // active rows (device scalar), or nullptr: Bmax
   const float* w_scale;     // FP8: [M]
   const float* x_scale;     // FP8: [Bmax]

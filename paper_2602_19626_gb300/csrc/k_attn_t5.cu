@@ -406,15 +406,16 @@ __global__ void __launch_bounds__(kT5Threads) k_attn_merge(Dims D, Batch b, int 
 // Prefill append: row j's k (rotated at its position a) and v, rounded to
 // BF16, into the ring of `layer`, and its query heads, rotated, scaled by 1/8
 // and rounded to BF16, into q16 (the attention's decode step does the same
-// arithmetic for its one row).  Sixteen threads take a row, thread i the
-// rotation pairs 2 i and 2 i + 1 of every head, so a position's rotations are
+// arithmetic for its one row).  A warp takes a row, lane i mod 16 the rotation
+// pairs 2 i and 2 i + 1 of every second head, so a position's rotations are
 // formed once and all heads' loads are in flight together (a CTA per row and
 // KV head took 13.8 us for 3,072 rows, most of it waiting).
-constexpr int kAppendThreads = 128, kAppendRows = kAppendThreads / 16;
+constexpr int kAppendThreads = 128, kAppendRows = kAppendThreads / 32;
 template <int HQ, int HKV>
 __global__ void __launch_bounds__(kAppendThreads) k_kv_append_t5(Dims D, Batch b, int layer, const float* qkv) {
   const int hq = HQ ? HQ : D.hq, hkv = HKV ? HKV : D.hkv;
-  const int j = blockIdx.x * kAppendRows + (threadIdx.x >> 4), dd = 2 * (threadIdx.x & 15);
+  const int j = blockIdx.x * kAppendRows + (threadIdx.x >> 5), dd = 2 * (threadIdx.x & 15);
+  const int half = (threadIdx.x >> 4) & 1;
   pdl_wait();
   pdl_trigger();
   if (j >= *b.nB) return;
@@ -429,7 +430,9 @@ __global__ void __launch_bounds__(kAppendThreads) k_kv_append_t5(Dims D, Batch b
   const float2 c0 = rope_cs(D, a, dd), c1 = rope_cs(D, a, dd + 1);
   auto put = [](__nv_bfloat16* dst, float x, float y) { *reinterpret_cast<uint32_t*>(dst) = pack_bf16(x, y); };
 #pragma unroll
-  for (int h = 0; h < hq + hkv; ++h) {             // the query heads, then the keys
+  for (int i = 0; i < (hq + hkv + 1) / 2; ++i) {   // the query heads, then the keys
+    const int h = 2 * i + half;
+    if (h >= hq + hkv) break;
     const float* src = row + h * kHeadDim + dd;
     const float2 x = __ldcg(reinterpret_cast<const float2*>(src));
     const float2 y = __ldcg(reinterpret_cast<const float2*>(src + kHeadDim / 2));
@@ -444,7 +447,9 @@ __global__ void __launch_bounds__(kAppendThreads) k_kv_append_t5(Dims D, Batch b
     }
   }
 #pragma unroll
-  for (int h = 0; h < hkv; ++h) {
+  for (int i = 0; i < (hkv + 1) / 2; ++i) {
+    const int h = 2 * i + half;
+    if (h >= hkv) break;
     const float4 v = __ldcg(reinterpret_cast<const float4*>(row + (hq + hkv + h) * kHeadDim + 2 * dd));
     *reinterpret_cast<uint2*>(ring + (size_t)(hkv + h) * plane + 2 * dd) =
         make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));

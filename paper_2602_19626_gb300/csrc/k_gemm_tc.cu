@@ -323,6 +323,7 @@ cudaError_t prepare_tc_epi() {
   if (e == cudaSuccess) e = prepare_tc_t<64, 8, KB, EPI, 1, 1>();
   if (e == cudaSuccess) e = prepare_tc_t<128, 6, KB, EPI, 1, 1>();
   if (e == cudaSuccess) e = prepare_tc_t<256, 4, KB, EPI, 1, 1>();
+  if (e == cudaSuccess) e = prepare_tc_t<32, 5, KB, EPI, 1, 2>();
   if (e == cudaSuccess) e = prepare_tc_t<64, 4, KB, EPI, 1, 2>();
   if (e == cudaSuccess) e = prepare_tc_t<128, 3, KB, EPI, 1, 2>();
   if (KB) {
@@ -358,6 +359,7 @@ cudaError_t launch_tc_epi(const TcGemm& g, cudaStream_t s, bool pdl) {
   if (g.kp == 2) return cudaErrorInvalidValue;
   if (g.occ == 2) {
     switch (g.bn) {
+      case 32: return launch_tc_t<32, 5, KB, EPI, 1, 2>(g, s, pdl);
       case 64: return launch_tc_t<64, 4, KB, EPI, 1, 2>(g, s, pdl);
       case 128: return launch_tc_t<128, 3, KB, EPI, 1, 2>(g, s, pdl);
     }
