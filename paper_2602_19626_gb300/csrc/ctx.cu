@@ -2127,8 +2127,8 @@ extern "C" int nc_decode(nc_ctx* ctx, const uint8_t* in, size_t nbytes, int32_t*
     }
     // one decode step (the decoder learns each token from the coder between
     // steps): the active count and the coder targets in from pinned host
-    // memory, the model, the CDFs, the search, the updates, the coded
-    // intervals and tokens out.  Captured once in a CUDA graph and replayed
+    // memory, the model, the counts, the target's symbol and the updates, the
+    // coded intervals and tokens out.  Captured once in a CUDA graph and replayed
     // per position; the copies read and write the same pinned buffers.
     uint32_t* h_in = ctx->h_u32;
     uint32_t* h_out = ctx->h_u32 + 1 + ctx->cfg.max_streams;
@@ -2139,14 +2139,13 @@ extern "C" int nc_decode(nc_ctx* ctx, const uint8_t* in, size_t nbytes, int32_t*
       cudaError_t e = cudaMemcpyAsync(ctx->d_dec_in, h_in, (1 + (size_t)n) * 4, cudaMemcpyHostToDevice, s);
       if (e == cudaSuccess) e = launch_model(ctx, b);
       VocabIO io{};
-      io.cdf = ctx->cdf;
       io.predict = 1;
+      io.update = 1;
+      io.ngram = 1;
+      io.target = ctx->d_dec_in + 1;
+      io.found = obs;
+      io.lohi = ctx->d_dec_out;
       if (e == cudaSuccess) e = launch_vocab(D, b, io, s);
-      if (e == cudaSuccess) e = launch_search(b, D.V, ctx->cdf, ctx->d_dec_in + 1, obs, ctx->d_dec_out, D.pdl, s);
-      VocabIO up{};
-      up.update = 1;
-      up.ngram = 1;
-      if (e == cudaSuccess) e = launch_vocab(D, b, up, s);
       if (e == cudaSuccess) e = cudaMemcpyAsync(h_out, ctx->d_dec_out, (size_t)n * 12, cudaMemcpyDeviceToHost, s);
       return e;
     };
@@ -2347,7 +2346,20 @@ extern "C" int nc_gemm_tc(const void* W, const void* X, const float* w_scale, co
   TcMat t;
   t.M = M;
   t.K = K;
-  if (!tc_encode_weights(t, W, esz) || !tc_encode_operand(t, &t.b[0][0], X, esz, N, bn)) return NC_EINVAL;
+  // Two CTAs per SM where there are tiles for them (the tuner's choice for
+  // such shapes): one's epilogue beside the other's loads.  Below two tiles
+  // per SM the deeper ring of one CTA is the faster.
+  int n_sm = 0, dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return NC_ECUDA;
+  const bool two = bn <= 128 && (int64_t)((M + 127) / 128) * ((N + bn - 1) / bn) >= 2 * (int64_t)n_sm;
+  if (two) {
+    t.kp = 1;
+    if (!tc_encode_tmap(&t.a, W, esz, K, M, 128) || !tc_encode_tmap(&t.b[0][0], X, esz, K, N, bn)) return NC_EINVAL;
+  } else if (!tc_encode_weights(t, W, esz) || !tc_encode_operand(t, &t.b[0][0], X, esz, N, bn)) {
+    return NC_EINVAL;
+  }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   WordLease w;
   const cudaError_t e = w.take();
@@ -2360,6 +2372,7 @@ extern "C" int nc_gemm_tc(const void* W, const void* X, const float* w_scale, co
   g.Bmax = N;
   g.bn = bn;
   g.kp = t.kp;
+  g.occ = two ? 2 : 1;
   g.kind_bf16 = !fp8;
   g.w_scale = w_scale;
   g.x_scale = x_scale;

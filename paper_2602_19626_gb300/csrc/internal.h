@@ -245,6 +245,12 @@ struct VocabIO {
   int predict;              // quantise (and write cdf / intervals)
   int update;               // apply head + mixer update with b.obs
   int ngram;                // with update: also the N-gram update and the stream's bookkeeping
+  // Decoder (predict and update set, b.obs null or not read): row j's token is
+  // the symbol whose counts hold target[j]; written to found[j], its interval
+  // to lohi[2 j], and the updates made with it.
+  const uint32_t* target;
+  int32_t* found;
+  uint32_t* lohi;
 };
 cudaError_t launch_vocab(const Dims& D, const Batch& b, const VocabIO& io, cudaStream_t s);
 // The vocabulary passes of a prefill chunk in one launch: stream row j runs
@@ -302,10 +308,6 @@ cudaError_t launch_gather_status(StreamDev* st, const int32_t* slots, int n, con
 cudaError_t launch_kv_append_t5(const Dims& D, const Batch& b, int layer, const float* qkv, cudaStream_t s);
 // Prefill: rotate and append the k, v of every row to the KV ring of `layer`.
 cudaError_t launch_kv_append(const Dims& D, const Batch& b, int layer, const float* qkv, cudaStream_t s);
-// Decoder: row j's symbol is the s with cdf[s] <= target[j] < cdf[s+1]; writes
-// obs[j] = s and lohi[2j..2j+1] = (cdf[s], cdf[s+1]).
-cudaError_t launch_search(const Batch& b, int V, const uint32_t* cdf, const uint32_t* target,
-                          int32_t* obs, uint32_t* lohi, bool pdl, cudaStream_t s);
 cudaError_t launch_convert_weights(const float* src, void* dst, float* scale, int64_t rows,
                                    int64_t cols, int fmt, cudaStream_t s);
 cudaError_t launch_interleave_f32(const float* gate, const float* up, float* dst, int64_t rows,
