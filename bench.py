@@ -92,10 +92,10 @@ BATCHED = ("batched_bf16_tc", "fp8_tc_1024x1024")
 
 
 # Kernels of one decode step on the tensor-core path with BF16 weights: the
-# embedding; per layer the RMSNorm operand, QKV, attention (with the append),
-# O, RMSNorm operand, gate/up and down; the final RMSNorm operand, the LM
-# head; the vocabulary step and the coder's device search.
-DECODE_STEP_LAUNCHES = 1 + 7 * 30 + 2 + 2
+# embedding; per layer QKV (with its RMSNorm), attention (with the append), O,
+# gate/up (with its RMSNorm) and down; the final RMSNorm operand, the LM head;
+# the vocabulary step (with the symbol search and the update).
+DECODE_STEP_LAUNCHES = 1 + 5 * 30 + 2 + 1
 
 
 def dist_env():
@@ -354,7 +354,7 @@ def ncu_traffic(kind: str, workload: str):
 # The device sources each traced kernel kind is built from; a kind not listed
 # is keyed by every device source.
 KIND_SOURCES = {
-    "attn": ("k_attn_t5.cu", "model_dev.cuh", "tc5.cuh", "internal.h"),
+    "attn": ("k_attn_t5.cu", "attn_t5.cuh", "model_dev.cuh", "tc5.cuh", "internal.h"),
     "vocab": ("k_vocab.cu", "internal.h"),
     "ngram_update": ("k_vocab.cu", "internal.h"),
 }

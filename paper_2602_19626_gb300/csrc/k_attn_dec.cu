@@ -307,9 +307,7 @@ cudaError_t launch_dec_s(const Dims& D, const Batch& b, int layer, const AttnIO&
 }  // namespace
 
 cudaError_t prepare_attn_dec() {
-  static bool done = false;                        // per-kernel attributes: once per process
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = cudaSuccess;                     // attributes of the current device's kernels
   auto set = [&](auto kern) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmem);
   };
@@ -317,7 +315,6 @@ cudaError_t prepare_attn_dec() {
   set(k_attn_dec<2>);
   set(k_attn_dec<4>);
   set(k_attn_dec<8>);
-  done = e == cudaSuccess;
   return e;
 }
 

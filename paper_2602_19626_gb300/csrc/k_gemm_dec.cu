@@ -296,9 +296,7 @@ bool gemm_dec_fits(int kind_bf16, int K, int pro) {
 }
 
 cudaError_t prepare_dec_kernels() {
-  static bool done = false;                        // per-kernel attributes: once per process
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaSuccess;
+  cudaError_t e = cudaSuccess;                     // attributes of the current device's kernels
   auto also = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
   for (int kb = 0; kb < 2; ++kb)
     for (int epi : {(int)EPI_STORE, (int)EPI_SWIGLU})
@@ -311,7 +309,6 @@ cudaError_t prepare_dec_kernels() {
   also(dec_prepare_t<1, EPI_RESID, DPRO_TMA, 32, 8, 1>());
   also(dec_prepare_t<0, EPI_RESID, DPRO_FP8, 32, 8, 1>());
   also(dec_prepare_t<0, EPI_RESID, DPRO_FP8, 32, 16, 1>());
-  done = e == cudaSuccess;
   return e;
 }
 

@@ -83,3 +83,33 @@ def test_mixed_nll_non_finite_rows():
                warm=torch.ones(4, dtype=torch.int32, device="cuda"))
     loss = mixed_nll(**arg)
     assert torch.isnan(loss[:3]).all() and torch.isfinite(loss[3])
+
+
+@pytest.mark.parametrize("fp8,K", [(False, 192), (False, 200), (True, 208)])
+def test_gemm_two_ctas_per_sm_equals_one(fp8, K):
+    """From two tiles per SM on, nc_gemm_tc runs two CTAs per SM (bn up to
+    128); bn 256 and few rows take one.  Every output accumulates its K blocks
+    in one order, so the results are equal, ragged edges included."""
+    import torch
+    from paper_2602_19626_gb300 import nc24 as nc
+    M, N = 1303, 3601                                # 11 x 29 tiles at bn 128
+    g = torch.Generator(device="cuda").manual_seed(K)
+    W = torch.randn(M, K, generator=g, device="cuda")
+    X = torch.randn(N, K, generator=g, device="cuda")
+    sc = dict(w_scale=None, x_scale=None)
+    if fp8:
+        sc = dict(w_scale=W.abs().amax(1) / 448, x_scale=X.abs().amax(1) / 448)
+        W, X = (W / sc["w_scale"][:, None]).to(torch.float8_e4m3fn), (X / sc["x_scale"][:, None]).to(torch.float8_e4m3fn)
+    else:
+        W, X = W.to(torch.bfloat16), X.to(torch.bfloat16)
+    ref = torch.empty(N, M, device="cuda")
+    assert nc.nc_gemm_tc(W, X, ref, bn=256, fp8=fp8, **sc) == nc.NC_OK
+    for bn in (32, 64, 128):
+        Y = torch.full((N, M), float("nan"), device="cuda")
+        assert nc.nc_gemm_tc(W, X, Y, bn=bn, fp8=fp8, **sc) == nc.NC_OK
+        assert torch.equal(Y, ref), bn
+    few = torch.empty(65, M, device="cuda")
+    if fp8:
+        sc["x_scale"] = sc["x_scale"][:65].contiguous()
+    assert nc.nc_gemm_tc(W, X[:65].contiguous(), few, bn=128, fp8=fp8, **sc) == nc.NC_OK
+    assert torch.equal(few, ref[:65])
