@@ -572,12 +572,17 @@ cudaError_t launch_gemv(const Dims& D, const Batch& b, const Mat& m, int fmt, in
   return gemv_f<NC_FP8E4M3>(D, b, m, pro, epi, io, s);
 }
 
-// CTAs per (row, KV head): the largest of 8, 4, 2, 1 that keeps the launch
-// within about two waves of two CTAs per SM.  Results do not depend on it.
+// CTAs per (row, KV head): as many as the longest window the launch may hold
+// has chunks (a power of two; 16 steps of the small FP32 model 2.52 -> 2.47 ms with
+// one CTA for windows of one chunk instead of eight), less where that keeps
+// the launch within about two waves of two CTAs per SM.  Results do not
+// depend on it.
 static int attn_split(const Dims& D, const Batch& b) {
   if (D.attn_cluster) return D.attn_cluster;
+  const int64_t len = b.len_max > 0 && b.len_max < D.L ? b.len_max : D.L;
+  const int nch = (int)((len + kAttnChunk - 1) / kAttnChunk);
   int S = 8;
-  while (S > 1 && (int64_t)D.hkv * b.Bmax * S > 4 * (int64_t)D.n_sm) S /= 2;
+  while (S > 1 && (S / 2 >= nch || (int64_t)D.hkv * b.Bmax * S > 4 * (int64_t)D.n_sm)) S /= 2;
   return S;
 }
 
