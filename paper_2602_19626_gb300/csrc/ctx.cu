@@ -2249,33 +2249,40 @@ extern "C" int nc_launch_chain_floor(int device, int n_links, int blocks, int th
 // for the length of a call, so that calls on several threads, streams and
 // devices each have their own and none allocates (a cudaMalloc and cudaFree
 // cost more than the kernels).  A word is zero when it is leased; a call that
-// raised it clears it, and one that failed to read it keeps it out of use.
-// With every word leased a call allocates its own.
+// raised it clears it, and one that failed to read it (the device's context is
+// lost) keeps it out of use.  With every word leased a call allocates its own,
+// cleared in the order of the call's stream.  A stream that is being captured
+// is refused before anything is put on it: the call has to wait for its status.
 static __device__ int32_t g_words[256];
 namespace {
 constexpr int kWords = 256, kWordDevices = 64;
+struct WordPool {
+  bool init = false;
+  int n = 0;                                       // free words
+  int free_word[kWords];
+};
 std::mutex g_words_mu;
-std::vector<int> g_words_free[kWordDevices];
-bool g_words_init[kWordDevices] = {};
+WordPool g_words_pool[kWordDevices];
 
 struct WordLease {
   int dev = -1, slot = -1;
   int32_t* p = nullptr;
   bool owned = false;                              // allocated by this call
-  cudaError_t take() {
-    cudaError_t e = cudaGetDevice(&dev);
+  cudaError_t take(cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &cap);
+    if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < kWordDevices) {
       std::lock_guard<std::mutex> lock(g_words_mu);
-      auto& f = g_words_free[dev];
-      if (!g_words_init[dev]) {
-        for (int i = 0; i < kWords; ++i) f.push_back(i);
-        g_words_init[dev] = true;
+      WordPool& f = g_words_pool[dev];
+      if (!f.init) {
+        for (int i = 0; i < kWords; ++i) f.free_word[i] = i;
+        f.n = kWords;
+        f.init = true;
       }
-      if (!f.empty()) {
-        slot = f.back();
-        f.pop_back();
-      }
+      if (f.n > 0) slot = f.free_word[--f.n];
     }
     void* q = nullptr;
     if (slot >= 0) {
@@ -2284,9 +2291,13 @@ struct WordLease {
       else give();
       return e;
     }
-    owned = true;
     e = dev_malloc(&p, 4);
-    return e == cudaSuccess ? cudaMemset(p, 0, 4) : e;
+    if (e != cudaSuccess) return e;
+    owned = true;
+    // on s: the legacy stream's order would not bind a non-blocking s
+    e = cudaMemsetAsync(p, 0, 4, s);
+    if (e != cudaSuccess) give();
+    return e;
   }
   // Read the word after the work on s, clear it if raised, give it back.
   cudaError_t finish(cudaStream_t s, int32_t* out) {
@@ -2305,7 +2316,8 @@ struct WordLease {
       cudaFree(p);
     } else if (slot >= 0) {
       std::lock_guard<std::mutex> lock(g_words_mu);
-      g_words_free[dev].push_back(slot);
+      WordPool& f = g_words_pool[dev];
+      f.free_word[f.n++] = slot;
     }
     slot = -1;
     owned = false;
@@ -2320,7 +2332,7 @@ extern "C" int nc_probs_to_cdf(const float* p, int n, int V, int log2_total, uin
     return NC_EINVAL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   WordLease w;
-  const cudaError_t e = w.take();
+  const cudaError_t e = w.take(s);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? NC_ENOMEM : NC_ECUDA;
   const cudaError_t el = launch_probs_to_cdf(p, n, V, log2_total, floor_c, cdf, w.p, false, s);
   int32_t bad = 0;
@@ -2364,7 +2376,7 @@ extern "C" int nc_gemm_tc(const void* W, const void* X, const float* w_scale, co
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   WordLease w;
-  const cudaError_t e = w.take();
+  const cudaError_t e = w.take(s);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? NC_ENOMEM : NC_ECUDA;
   TcGemm g{};
   g.tmap_a = &t.a;
