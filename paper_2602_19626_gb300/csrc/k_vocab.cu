@@ -1844,100 +1844,78 @@ __global__ void k_floor_counts(const float* p, int64_t n, uint32_t K, uint32_t f
   }
 }
 
-// Mixed-distribution NLL forward / backward, one CTA of NT threads per row.
+// Mixed-distribution NLL forward / backward, one CTA per row.  Thread t takes
+// symbols t, t + 512, .. in increasing order for the softmax's sum, the warps
+// the xor tree, then the warps in order, whatever the batch, the row's place
+// in it and its alignment: a row alone has the bits it has in any batch.
 //
-// Bound by memory: the softmax's maximum and sum come from one pass (each
-// thread keeps a running maximum and rescales its sum when it rises), four
-// values a load where the rows allow it, so the forward reads z and b once
-// from HBM and the backward's second pass finds them in L2.  The first
-// version made a pass for the maximum and a pass for the sum, one value a
-// load: 113 us each way for 512 rows of 49,152 (201 MB in, backward 101 MB out).
-constexpr int kNllVec = 4;                         // vectors of four in flight per array
+// Bound by memory at many rows: a pass for the maximum, one for the sum and
+// (backward) one for the gradient, each starting with the symbols that the
+// pass before read last, so that part of a row is found in L2.  Measured
+// (GB300, 512 rows of 49,152: 201 MB in, backward 101 MB out): forward 52 us,
+// backward 98; of 50,001: 56 and 105.  With four values ahead instead of
+// eight 57 and 107, with a row's scores kept in shared memory (one CTA per SM)
+// 89 and 128; one value a load without the order of the passes 69 and 159.
+constexpr int kNllThreads = 512;
+constexpr int kNllAhead = 8;                       // values of each array in flight per thread
 
-// fn(v, z_v, b_v) for the row's symbols in steps of the block; `vec`: 16-byte
-// aligned rows.
-template <int NT, typename F>
-__device__ __forceinline__ void nll_pass(const float* zr, const float* br, int V, bool vec, F fn) {
-  int done = 0;
-  if (vec) {
-    const int nv = V / 4;
-    for (int q0 = threadIdx.x; q0 < nv; q0 += NT * kNllVec) {
-      float4 zv[kNllVec], bv[kNllVec];
+// fn(v, z_v, b_v) for the thread's symbols, upwards or DOWN.
+template <bool DOWN, typename F>
+__device__ __forceinline__ void nll_pass(const float* zr, const float* br, int V, F fn) {
+  const int n = (V - 1 - (int)threadIdx.x + kNllThreads) / kNllThreads;   // symbols of the thread, 0 or more
+  const int step = DOWN ? -kNllThreads : kNllThreads;
+  int v = (int)threadIdx.x + (DOWN ? kNllThreads * (n - 1) : 0), i = 0;
+  for (; i + kNllAhead <= n; i += kNllAhead, v += kNllAhead * step) {
+    float z[kNllAhead], b[kNllAhead];
 #pragma unroll
-      for (int k = 0; k < kNllVec; ++k)
-        if (q0 + NT * k < nv) {
-          zv[k] = __ldg(reinterpret_cast<const float4*>(zr) + q0 + NT * k);
-          bv[k] = __ldg(reinterpret_cast<const float4*>(br) + q0 + NT * k);
-        }
-#pragma unroll
-      for (int k = 0; k < kNllVec; ++k)
-        if (q0 + NT * k < nv) fn(4 * (q0 + NT * k), zv[k], bv[k], 4);
+    for (int k = 0; k < kNllAhead; ++k) {
+      z[k] = zr[v + k * step];
+      b[k] = br[v + k * step];
     }
-    done = 4 * nv;
+#pragma unroll
+    for (int k = 0; k < kNllAhead; ++k) fn(v + k * step, z[k], b[k]);
   }
-  for (int v = done + threadIdx.x; v < V; v += NT)
-    fn(v, make_float4(zr[v], 0.f, 0.f, 0.f), make_float4(br[v], 0.f, 0.f, 0.f), 1);
+  for (; i < n; ++i, v += step) fn(v, zr[v], br[v]);
 }
 
-template <int NT>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(kNllThreads)
     k_mix_nll(const float* z, const float* bv, const float* png, const float* theta,
               const int32_t* target, const int32_t* warm, const float* gout, int V, float tau,
               float* loss, float* db, float* dth) {
-  __shared__ float2 part[NT / 32];
+  __shared__ float wmax[kNllThreads / 32], wsum[kNllThreads / 32];
   const int j = blockIdx.x;
   const float* zr = z + (size_t)j * V;
   const float* br = bv + (size_t)j * V;
   float* dr = db ? db + (size_t)j * V : nullptr;
   const int t = target[j];
   if (t < 0 || t >= V) {     // out-of-range target: NaN loss and gradients
-    for (int v = threadIdx.x; v < V && dr; v += NT) dr[v] = NAN;
+    for (int v = threadIdx.x; v < V && dr; v += kNllThreads) dr[v] = NAN;
     if (threadIdx.x == 0) {
       if (loss) loss[j] = NAN;
       if (dth) dth[2 * j] = dth[2 * j + 1] = NAN;
     }
     return;
   }
-  const bool vec = ((reinterpret_cast<uintptr_t>(zr) | reinterpret_cast<uintptr_t>(br) |
-                     reinterpret_cast<uintptr_t>(dr)) & 15) == 0;
   // s = z / tau + b as the coding step forms it (Sec. 3.2, Sec. 3.6): one
   // fused multiply-add by the rounded reciprocal of tau
   const float inv_tau = 1.0f / tau;
   auto score = [&](float zz, float bb) { return __fmaf_rn(zz, inv_tau, bb); };
-  float m = -INFINITY, ls = 0.f;
-  // (m, ls) <- merged with another maximum and sum; while a maximum is -inf
-  // its sum is 0, or NaN if a NaN was seen
-  auto add = [&](float mx, float sum) {
-    if (mx > m) {
-      ls = (m == -INFINITY ? ls : ls * expf(m - mx)) + sum;
-      m = mx;
-    } else {
-      ls += mx == m || mx == -INFINITY ? sum : sum * expf(mx - m);
-    }
-  };
-  nll_pass<NT>(zr, br, V, vec, [&](int, float4 a, float4 b, int n) {
-    const float s0 = score(a.x, b.x);
-    if (n == 1) {                                  // exp(s0 - s0): 1, or NaN for an infinite or NaN score
-      add(s0, s0 == -INFINITY ? 0.f : expf(s0 - s0));
-      return;
-    }
-    const float s1 = score(a.y, b.y), s2 = score(a.z, b.z), s3 = score(a.w, b.w);
-    const float mx = fmaxf(fmaxf(s0, s1), fmaxf(s2, s3));
-    if (mx > m) {
-      if (m > -INFINITY) ls *= expf(m - mx);
-      m = mx;
-    }
-    if (m > -INFINITY) ls += (expf(s0 - m) + expf(s1 - m)) + (expf(s2 - m) + expf(s3 - m));
-    else if (s0 != s0 || s1 != s1 || s2 != s2 || s3 != s3) ls = NAN;
-  });
-#pragma unroll
-  for (int o = 16; o; o >>= 1) add(__shfl_xor_sync(0xffffffffu, m, o), __shfl_xor_sync(0xffffffffu, ls, o));
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_float2(m, ls);
+  // the maximum in decreasing order of the symbols, so that the sum's pass
+  // starts with what it read last
+  float m = -INFINITY;
+  nll_pass<true>(zr, br, V, [&](int, float a, float b) { m = fmaxf(m, score(a, b)); });
+  m = warp_max(m);
+  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
   __syncthreads();
-  m = part[0].x;
-  ls = part[0].y;
-  for (int i = 1; i < NT / 32; ++i) add(part[i].x, part[i].y);
-  const float M = m, S = m == -INFINITY ? NAN : ls;
+  float M = wmax[0];
+  for (int i = 1; i < kNllThreads / 32; ++i) M = fmaxf(M, wmax[i]);
+  float ls = 0.f;
+  nll_pass<false>(zr, br, V, [&](int, float a, float b) { ls += expf(score(a, b) - M); });
+  ls = warp_sum(ls);
+  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = ls;
+  __syncthreads();
+  float S = 0.f;
+  for (int i = 0; i < kNllThreads / 32; ++i) S += wsum[i];
   const float pts = __fdiv_rn(expf(score(zr[t], br[t]) - M), S);
   const float pngs = png[(size_t)j * V + t];
   const float th0 = theta[2 * j], th1 = theta[2 * j + 1];
@@ -1950,16 +1928,9 @@ __global__ void __launch_bounds__(NT)
   if (loss && threadIdx.x == 0) loss[j] = -logf(pm);
   if (dr) {
     const float rho = wu ? 1.f : w0 * pts / pm;
-    auto grad = [&](float zz, float bb, int v) {
-      const float ptv = __fdiv_rn(expf(score(zz, bb) - M), S);
-      return g * rho * (ptv - (v == t ? 1.f : 0.f));
-    };
-    nll_pass<NT>(zr, br, V, vec, [&](int v, float4 a, float4 b, int n) {
-      if (n == 1)
-        dr[v] = grad(a.x, b.x, v);
-      else
-        __stcs(reinterpret_cast<float4*>(dr + v), make_float4(grad(a.x, b.x, v), grad(a.y, b.y, v + 1),
-                                                              grad(a.z, b.z, v + 2), grad(a.w, b.w, v + 3)));
+    nll_pass<true>(zr, br, V, [&](int v, float a, float b) {
+      const float ptv = __fdiv_rn(expf(score(a, b) - M), S);
+      dr[v] = g * rho * (ptv - (v == t ? 1.f : 0.f));
     });
   }
   if (dth && threadIdx.x == 0) {
@@ -2206,11 +2177,7 @@ cudaError_t launch_mix_nll(const float* z, const float* b, const float* png, con
                            const int32_t* target, const int32_t* warm, const float* gout, int n,
                            int V, float tau, float* loss, float* db, float* dtheta,
                            cudaStream_t s) {
-  // few rows: more threads per row; many: two CTAs per SM
-  if (n <= 152)
-    k_mix_nll<1024><<<n, 1024, 0, s>>>(z, b, png, theta, target, warm, gout, V, tau, loss, db, dtheta);
-  else
-    k_mix_nll<512><<<n, 512, 0, s>>>(z, b, png, theta, target, warm, gout, V, tau, loss, db, dtheta);
+  k_mix_nll<<<n, kNllThreads, 0, s>>>(z, b, png, theta, target, warm, gout, V, tau, loss, db, dtheta);
   return cudaGetLastError();
 }
 
