@@ -778,7 +778,7 @@ extern "C" int nc_ctx_create(const nc_config* cfg, const void* weights, size_t n
   if (D.kv_bf16) {
     D.attn_part_cap = attn_t5_scratch(D, ctx->P);
     if (ctx->P > 0 && dalloc(ctx, &D.attn_part, D.attn_part_cap * 4)) return bail(NC_ENOMEM);
-    if (prepare_attn_dec() != cudaSuccess) return bail(NC_ECUDA);
+    if (prepare_attn_dec() != cudaSuccess || prepare_attn_t5() != cudaSuccess) return bail(NC_ECUDA);
     if (ctx->P > 0 && dalloc(ctx, &D.q16, (size_t)ctx->P * D.hq * kHeadDim * 2)) return bail(NC_ENOMEM);
     // the attention loads 64-row boxes of the KV rings through one TMA map per slot
     void* maps = nullptr;
@@ -794,7 +794,7 @@ extern "C" int nc_ctx_create(const nc_config* cfg, const void* weights, size_t n
   ctx->slots.assign(B, Slot{});
   if (cudaMemset(ctx->d_st, 0, B * sizeof(StreamDev)) != cudaSuccess) return bail(NC_ECUDA);
   if (cudaMemset(ctx->d_status, 0, B * 4) != cudaSuccess) return bail(NC_ECUDA);
-  if (prepare_model_kernels(D, ctx->fmt) != cudaSuccess || prepare_vocab_kernels(D) != cudaSuccess ||
+  if (prepare_model_kernels(D, ctx->fmt) != cudaSuccess || prepare_vocab_kernels(&D) != cudaSuccess ||
       (c.path == NC_PATH_TC && (prepare_tc_kernels() != cudaSuccess || prepare_dec_kernels() != cudaSuccess)))
     return bail(NC_ECUDA);
   if (c.path == NC_PATH_TC) {
@@ -2351,7 +2351,6 @@ extern "C" int nc_gemm_tc(const void* W, const void* X, const float* w_scale, co
                           int N, int K, int bn, float* Y, void* stream) {
   if (!W || !X || !Y || M < 1 || N < 1 || K < 1 || (fp8 && (!w_scale || !x_scale))) return NC_EINVAL;
   cudaGetLastError();                              // a stale error of an earlier call is not ours
-  if (prepare_tc_kernels() != cudaSuccess) return NC_ECUDA;
   if (bn != 32 && bn != 64 && bn != 128 && bn != 256) return NC_EINVAL;
   const int esz = fp8 ? 1 : 2;
   if ((K * esz) % 16 || (reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(X)) % 16) return NC_EINVAL;
@@ -2392,7 +2391,8 @@ extern "C" int nc_gemm_tc(const void* W, const void* X, const float* w_scale, co
   g.x_scale = x_scale;
   g.y = Y;
   g.status = w.p;
-  const cudaError_t el = launch_gemm_tc(g, EPI_STORE, s, false);
+  cudaError_t el = prepare_gemm_store(g);
+  if (el == cudaSuccess) el = launch_gemm_tc(g, EPI_STORE, s, false);
   int32_t gave_up = 0;
   const cudaError_t ef = w.finish(s, &gave_up);
   if (el != cudaSuccess || ef != cudaSuccess) return NC_ECUDA;

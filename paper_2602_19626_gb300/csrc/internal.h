@@ -84,6 +84,7 @@ struct Dims {
   int kv_bf16;              // 1: KV cache in BF16
   int attn_cluster;         // CTAs per (stream, KV head) in the FP32-cache attention: 1, 2, 4 or 8; 0 = by batch size
   int n_sm;                 // SMs of the device
+  int cl16;                 // clusters of 16 CTAs of the vocabulary kernels can be placed on it
   int order;                // N-gram order (0 = off)
   int skip;                 // confidence skip: p = p_ng when H(p_ng) < kSkipBits
   int use_head;
@@ -295,6 +296,7 @@ size_t attn_t5_scratch(const Dims& D, int prefill_rows);
 cudaError_t launch_attn_dec(const Dims& D, const Batch& b, int layer, const float* qkv, float* attn_out, void* out16,
                             cudaStream_t s);
 cudaError_t prepare_attn_dec();
+cudaError_t prepare_attn_t5();
 // log2 of its cluster size for the launch's rows (Batch::len_max).
 int attn_dec_class(const Dims& D, const Batch& b);
 // Fresh state of a stream: bias, unigram counts and the hash index cleared,
@@ -373,8 +375,9 @@ cudaError_t launch_act_plain(const Dims& D, const Batch& b, const float* x, int 
 // Kernel attributes (dynamic shared memory limits) set once, outside any
 // stream capture.
 cudaError_t prepare_model_kernels(const Dims& D, int fmt);
-cudaError_t prepare_vocab_kernels(const Dims& D);
+cudaError_t prepare_vocab_kernels(Dims* D);       // sets D->cl16
 cudaError_t prepare_tc_kernels();
+cudaError_t prepare_gemm_store(const TcGemm& g);   // of the variant that launch_gemm_tc(g, EPI_STORE) takes
 
 // status: a word per row (per_row), or one word that any bad row raises.
 cudaError_t launch_probs_to_cdf(const float* p, int n, int V, int log2T, uint32_t floor,

@@ -467,16 +467,14 @@ size_t attn_t5_scratch(const Dims& D, int prefill_rows) {
   return pf_pairs * (size_t)D.hkv * kT5MaxRanks * kPartRow;
 }
 
+cudaError_t prepare_attn_t5() {                    // the limit of the current device's context
+  return cudaFuncSetAttribute(k_attn_t5, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kT5Smem);
+}
+
 cudaError_t launch_attn_t5(const Dims& D, const Batch& b, int layer, const float* qkv, float* attn_out, void* out16,
                            cudaStream_t s) {
   if (!b.pos) return launch_attn_dec(D, b, layer, qkv, attn_out, out16, s);
   if (!D.attn_part || !D.q16) return cudaErrorInvalidValue;
-  static bool attr = false;                        // the kernel's shared-memory limit, once per process
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(k_attn_t5, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kT5Smem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
   const int grp = D.hq / D.hkv;
   if (grp > kT5Pairs) return cudaErrorInvalidValue;
   const int tps = (b.pm * grp + kT5Pairs - 1) / kT5Pairs, tiles = (b.Bmax / b.pm) * tps;

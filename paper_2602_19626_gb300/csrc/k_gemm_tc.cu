@@ -311,67 +311,78 @@ EncodeTiled encode_fn() {
   return fn;
 }
 
-template <int BN, int STAGES, int KB, int EPI, int KP, int OCC>
-cudaError_t prepare_tc_t() {
-  return cudaFuncSetAttribute(k_gemm_tc<BN, STAGES, KB, EPI, KP, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)tc_smem_bytes<BN, STAGES, KP>());
-}
+// A variant of the kernel: batch tile, pipeline stages, K blocks per stage,
+// CTAs per SM.
+template <int BN_, int STAGES_, int KP_, int OCC_>
+struct TcTile {
+  static constexpr int BN = BN_, STAGES = STAGES_, KP = KP_, OCC = OCC_;
+  static constexpr size_t smem = tc_smem_bytes<BN_, STAGES_, KP_>();
+};
 
-template <int KB, int EPI>
-cudaError_t prepare_tc_epi() {
-  cudaError_t e = prepare_tc_t<32, 10, KB, EPI, 1, 1>();
-  if (e == cudaSuccess) e = prepare_tc_t<64, 8, KB, EPI, 1, 1>();
-  if (e == cudaSuccess) e = prepare_tc_t<128, 6, KB, EPI, 1, 1>();
-  if (e == cudaSuccess) e = prepare_tc_t<256, 4, KB, EPI, 1, 1>();
-  if (e == cudaSuccess) e = prepare_tc_t<32, 5, KB, EPI, 1, 2>();
-  if (e == cudaSuccess) e = prepare_tc_t<64, 4, KB, EPI, 1, 2>();
-  if (e == cudaSuccess) e = prepare_tc_t<128, 3, KB, EPI, 1, 2>();
-  if (KB) {
-    if (e == cudaSuccess) e = prepare_tc_t<32, 5, KB, EPI, 2, 1>();
-    if (e == cudaSuccess) e = prepare_tc_t<64, 4, KB, EPI, 2, 1>();
-    if (e == cudaSuccess) e = prepare_tc_t<128, 3, KB, EPI, 2, 1>();
-    if (e == cudaSuccess) e = prepare_tc_t<256, 2, KB, EPI, 2, 1>();
-  }
-  return e;
-}
-
-template <int BN, int STAGES, int KB, int EPI, int KP, int OCC>
-cudaError_t launch_tc_t(const TcGemm& g, cudaStream_t s, bool pdl) {
-  constexpr size_t smem = tc_smem_bytes<BN, STAGES, KP>();
-  auto kern = k_gemm_tc<BN, STAGES, KB, EPI, KP, OCC>;
-  dim3 grid((g.M + kTileM - 1) / kTileM, (g.Bmax + BN - 1) / BN);
-  const CUtensorMap* a = reinterpret_cast<const CUtensorMap*>(g.tmap_a);
-  const CUtensorMap* b = reinterpret_cast<const CUtensorMap*>(g.tmap_b);
-  return launch_kernel(kern, grid, dim3(kTcThreads), smem, s, pdl, *a, *b, g);
-}
-
-template <int KB, int EPI>
-cudaError_t launch_tc_epi(const TcGemm& g, cudaStream_t s, bool pdl) {
-  if (KB && g.kp == 2 && g.K % 64 == 0) {
-    switch (g.bn) {
-      case 32: return launch_tc_t<32, 5, KB, EPI, 2, 1>(g, s, pdl);
-      case 64: return launch_tc_t<64, 4, KB, EPI, 2, 1>(g, s, pdl);
-      case 128: return launch_tc_t<128, 3, KB, EPI, 2, 1>(g, s, pdl);
-      case 256: return launch_tc_t<256, 2, KB, EPI, 2, 1>(g, s, pdl);
+// f(the variant g asks for).
+template <int KB, typename F>
+cudaError_t tc_pick(const TcGemm& g, F f) {
+  if constexpr (KB != 0) {
+    if (g.kp == 2 && g.K % 64 == 0) {
+      switch (g.bn) {
+        case 32: return f(TcTile<32, 5, 2, 1>());
+        case 64: return f(TcTile<64, 4, 2, 1>());
+        case 128: return f(TcTile<128, 3, 2, 1>());
+        case 256: return f(TcTile<256, 2, 2, 1>());
+      }
+      return cudaErrorInvalidValue;
     }
-    return cudaErrorInvalidValue;
   }
   if (g.kp == 2) return cudaErrorInvalidValue;
   if (g.occ == 2) {
     switch (g.bn) {
-      case 32: return launch_tc_t<32, 5, KB, EPI, 1, 2>(g, s, pdl);
-      case 64: return launch_tc_t<64, 4, KB, EPI, 1, 2>(g, s, pdl);
-      case 128: return launch_tc_t<128, 3, KB, EPI, 1, 2>(g, s, pdl);
+      case 32: return f(TcTile<32, 5, 1, 2>());
+      case 64: return f(TcTile<64, 4, 1, 2>());
+      case 128: return f(TcTile<128, 3, 1, 2>());
     }
     return cudaErrorInvalidValue;
   }
   switch (g.bn) {
-    case 32: return launch_tc_t<32, 10, KB, EPI, 1, 1>(g, s, pdl);
-    case 64: return launch_tc_t<64, 8, KB, EPI, 1, 1>(g, s, pdl);
-    case 128: return launch_tc_t<128, 6, KB, EPI, 1, 1>(g, s, pdl);
-    case 256: return launch_tc_t<256, 4, KB, EPI, 1, 1>(g, s, pdl);
+    case 32: return f(TcTile<32, 10, 1, 1>());
+    case 64: return f(TcTile<64, 8, 1, 1>());
+    case 128: return f(TcTile<128, 6, 1, 1>());
+    case 256: return f(TcTile<256, 4, 1, 1>());
   }
   return cudaErrorInvalidValue;
+}
+
+// The shared-memory limit of the variant g asks for, in the current device's
+// context (a limit holds for one context).
+template <int KB, int EPI>
+cudaError_t prepare_tc_one(const TcGemm& g) {
+  return tc_pick<KB>(g, [](auto t) {
+    using T = decltype(t);
+    return cudaFuncSetAttribute(k_gemm_tc<T::BN, T::STAGES, KB, EPI, T::KP, T::OCC>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem);
+  });
+}
+
+template <int KB, int EPI>
+cudaError_t prepare_tc_epi() {
+  cudaError_t e = cudaSuccess;
+  TcGemm g{};
+  g.K = 64;
+  for (g.kp = 1; g.kp <= (KB ? 2 : 1); ++g.kp)
+    for (g.occ = 1; g.occ <= 3 - g.kp; ++g.occ)
+      for (g.bn = 32; g.bn <= (g.occ == 2 ? 128 : 256) && e == cudaSuccess; g.bn *= 2) e = prepare_tc_one<KB, EPI>(g);
+  return e;
+}
+
+template <int KB, int EPI>
+cudaError_t launch_tc_epi(const TcGemm& g, cudaStream_t s, bool pdl) {
+  return tc_pick<KB>(g, [&](auto t) {
+    using T = decltype(t);
+    const dim3 grid((g.M + kTileM - 1) / kTileM, (g.Bmax + T::BN - 1) / T::BN);
+    const CUtensorMap* a = reinterpret_cast<const CUtensorMap*>(g.tmap_a);
+    const CUtensorMap* b = reinterpret_cast<const CUtensorMap*>(g.tmap_b);
+    return launch_kernel(k_gemm_tc<T::BN, T::STAGES, KB, EPI, T::KP, T::OCC>, grid, dim3(kTcThreads), T::smem, s, pdl,
+                         *a, *b, g);
+  });
 }
 
 // ------------------------------------------------- activation preparation
@@ -563,24 +574,19 @@ bool tc_encode_tmap(void* tmap, const void* base, int elem_bytes, int64_t inner,
 }
 
 cudaError_t prepare_tc_kernels() {
-  static bool done = false;                        // per-kernel attributes: once per process
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaSuccess;
-  for (int kb = 0; kb < 2 && e == cudaSuccess; ++kb) {
-    if (kb) {
-      e = prepare_tc_epi<1, EPI_STORE>();
-      if (e == cudaSuccess) e = prepare_tc_epi<1, EPI_RESID>();
-      if (e == cudaSuccess) e = prepare_tc_epi<1, EPI_SWIGLU>();
-      if (e == cudaSuccess) e = prepare_tc_epi<1, EPI_LOGITS>();
-    } else {
-      e = prepare_tc_epi<0, EPI_STORE>();
-      if (e == cudaSuccess) e = prepare_tc_epi<0, EPI_RESID>();
-      if (e == cudaSuccess) e = prepare_tc_epi<0, EPI_SWIGLU>();
-      if (e == cudaSuccess) e = prepare_tc_epi<0, EPI_LOGITS>();
-    }
-  }
-  done = e == cudaSuccess;
+  cudaError_t e = prepare_tc_epi<1, EPI_STORE>();
+  if (e == cudaSuccess) e = prepare_tc_epi<1, EPI_RESID>();
+  if (e == cudaSuccess) e = prepare_tc_epi<1, EPI_SWIGLU>();
+  if (e == cudaSuccess) e = prepare_tc_epi<1, EPI_LOGITS>();
+  if (e == cudaSuccess) e = prepare_tc_epi<0, EPI_STORE>();
+  if (e == cudaSuccess) e = prepare_tc_epi<0, EPI_RESID>();
+  if (e == cudaSuccess) e = prepare_tc_epi<0, EPI_SWIGLU>();
+  if (e == cudaSuccess) e = prepare_tc_epi<0, EPI_LOGITS>();
   return e;
+}
+
+cudaError_t prepare_gemm_store(const TcGemm& g) {
+  return g.kind_bf16 ? prepare_tc_one<1, EPI_STORE>(g) : prepare_tc_one<0, EPI_STORE>(g);
 }
 
 cudaError_t launch_gemm_tc(const TcGemm& g, int epi, cudaStream_t s, bool pdl) {

@@ -1984,15 +1984,12 @@ static bool step_full(int V) {
   return V == kClusterWarps * 32 * E;
 }
 
-// 16-CTA clusters (a non-portable size) are used when the device places them.
-static bool g_cl16 = false;
-
-// CTAs per stream of a step launch over `rows` streams: 16 while the
-// clusters fit in one wave (one stream or a few: the per-position latency
-// falls with the work per SM), else 8 (more streams per wave).  Results do
-// not depend on it.
+// CTAs per stream of a step launch over `rows` streams: 16 (a non-portable
+// cluster size, Dims::cl16) while the clusters fit in one wave (one stream or
+// a few: the per-position latency falls with the work per SM), else 8 (more
+// streams per wave).  Results do not depend on it.
 static int step_cluster(const Dims& D, int rows) {
-  return g_cl16 && rows * 16 <= D.n_sm ? 16 : 8;
+  return D.cl16 && rows * 16 <= D.n_sm ? 16 : 8;
 }
 
 template <int E, bool FULL, int CL>
@@ -2042,24 +2039,24 @@ static bool clusters_fit() {
   return ok;
 }
 template <int E, bool FULL>
-static cudaError_t prepare_vocab_tf() {
+static cudaError_t prepare_vocab_tf(Dims* D) {
   cudaError_t e = prepare_vocab_tfc<E, FULL, 8>();
   if (e != cudaSuccess) return e;
-  g_cl16 = prepare_vocab_tfc<E, FULL, 16>() == cudaSuccess && clusters_fit<E, FULL, 16>();
+  D->cl16 = prepare_vocab_tfc<E, FULL, 16>() == cudaSuccess && clusters_fit<E, FULL, 16>();
   cudaGetLastError();
   return cudaSuccess;
 }
 template <int E>
-static cudaError_t prepare_vocab_t(int V) {
-  return step_full<E>(V) ? prepare_vocab_tf<E, true>() : prepare_vocab_tf<E, false>();
+static cudaError_t prepare_vocab_t(Dims* D) {
+  return step_full<E>(D->V) ? prepare_vocab_tf<E, true>(D) : prepare_vocab_tf<E, false>(D);
 }
 
-cudaError_t prepare_vocab_kernels(const Dims& D) {
-  switch (vocab_E(D.V, 8, step_threads<8>())) {
-    case 4: return prepare_vocab_t<4>(D.V);
-    case 8: return prepare_vocab_t<8>(D.V);
-    case 12: return prepare_vocab_t<12>(D.V);
-    case 16: return prepare_vocab_t<16>(D.V);
+cudaError_t prepare_vocab_kernels(Dims* D) {
+  switch (vocab_E(D->V, 8, step_threads<8>())) {
+    case 4: return prepare_vocab_t<4>(D);
+    case 8: return prepare_vocab_t<8>(D);
+    case 12: return prepare_vocab_t<12>(D);
+    case 16: return prepare_vocab_t<16>(D);
   }
   return cudaErrorInvalidValue;
 }
