@@ -18,12 +18,8 @@ class MixedNLL(torch.autograd.Function):
         for t in (b, theta, z, p_ng):
             if not (t.is_cuda and t.dtype == torch.float32 and t.is_contiguous()):
                 raise ValueError("MixedNLL expects contiguous float32 CUDA tensors")
-        # as they are when they already are (the conversions cost some 10 us of
-        # host time each, and the call is host bound up to 512 rows)
-        if target.dtype != torch.int32 or not target.is_contiguous():
-            target = target.to(torch.int32).contiguous()
-        if warm.dtype != torch.int32 or not warm.is_contiguous():
-            warm = warm.to(torch.int32).contiguous()
+        target = target.to(torch.int32).contiguous()
+        warm = warm.to(torch.int32).contiguous()
         loss = torch.empty(z.shape[0], device=z.device, dtype=torch.float32)
         st = nc24.nc_mix_nll_fwd(z, b, p_ng, theta, target, warm, tau, loss)
         if st:
