@@ -259,7 +259,8 @@ const char* nc_last_error(const nc_ctx* ctx);
  * default stream).  Returns NC_ENUMERIC when a row holds a non-finite or
  * negative value, a value >= 2, or the residual would leave the argmax count
  * below the floor (that row's cdf is then unspecified); NC_EINVAL for bad
- * sizes.  Synchronises the stream. */
+ * sizes.  Synchronises the stream; a stream that is being captured is refused
+ * (NC_ECUDA, the capture goes on). */
 int nc_probs_to_cdf(const float* p, int n, int V, int log2_total, uint32_t floor,
                     uint32_t* cdf, void* stream);
 
@@ -313,7 +314,8 @@ int nc_stream_state(nc_ctx* ctx, int32_t stream_id, float* bias, float* mix_logw
  *   w_scale DEVICE float[M], x_scale DEVICE float[N] (FP8 only): the product
  *     is scaled by w_scale[m] * x_scale[n].
  *   bn: batch tile, 32 | 64 | 128 | 256 (results do not depend on it).
- *   Y DEVICE float[N][M].  Synchronises `stream`.
+ *   Y DEVICE float[N][M].  Synchronises `stream`; one that is being captured is
+ *     refused (NC_ECUDA, the capture goes on).
  * Errors: NC_EINVAL, NC_ENOMEM, NC_ECUDA, NC_ETIMEOUT (a bounded pipeline
  * wait gave up). */
 int nc_gemm_tc(const void* W, const void* X, const float* w_scale, const float* x_scale, int fp8, int M,

@@ -2357,11 +2357,13 @@ extern "C" int nc_gemm_tc(const void* W, const void* X, const float* w_scale, co
   TcMat t;
   t.M = M;
   t.K = K;
-  // Two CTAs per SM where there are tiles for them (the tuner's choice for
-  // such shapes): one's epilogue beside the other's loads.  Measured for the
-  // LM head over 1,024 rows (3,072 tiles): 154 us a call with one CTA per SM,
-  // 115 with two.  Below two tiles per SM there is no second tile to overlap
-  // and the deeper ring of one CTA serves it.
+  // Two CTAs per SM where there are tiles for them: one's epilogue beside the
+  // other's loads.  Below two tiles per SM there is no second tile to overlap
+  // and the deeper ring of one CTA serves it.  Measured (GB300, time of a call
+  // with one CTA per SM over that with two; M 576 to 4,096, K 576 to 3,072, bn
+  // 32 to 128, both formats): 256 tiles 0.91 to 1.01 in all but two, 320 and
+  // 384 tiles 0.94 to 1.2, 512 to 768 tiles 1.01 to 1.3, more 1.09 to 1.6;
+  // the LM head over 1,024 rows (3,072 tiles) 154 us and 115.
   int n_sm = 0, dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)

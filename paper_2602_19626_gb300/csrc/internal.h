@@ -170,10 +170,7 @@ __device__ __forceinline__ size_t kv_plane_off(int L, int hkv, int layer, int wh
 // no in-flight kernel writes (weights, KV entries of earlier tokens, state of
 // earlier steps) before pdl_wait(), and signals its own dependents only
 // after pdl_wait(); so when a kernel's pdl_wait() returns, every earlier
-// kernel of the stream has completed and its writes are visible.  (Signalling
-// before the wait too, so that several kernels' weights are in flight, was
-// tried on the decode step: 907 us a token against 854, the waiting CTAs'
-// traffic slowed the running kernel more than it hid.)
+// kernel of the stream has completed and its writes are visible.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -337,10 +334,18 @@ struct TcGemm {
 };
 // The projection of a decode step of at most kDecMaxRows rows (k_gemm_dec.cu):
 // the same products in the same order, with the operand made in the kernel.
-// The line is the row tile of its norm prologue: past 64 rows every CTA would
-// make more rows than the row kernel spreads over the whole chip.
+// Every CTA makes its rows itself, so this loses with the rows; the launch
+// knows the rows it may hold, not how many of them are still active.  Measured
+// (GB300, full model, one nc_step_probe, in us: this, then operand kernels and
+// k_gemm_tc):
+//   BF16   8 rows 551, 784; 32: 709, 819; 48: 849, 843; 64: 907, 862; 96: 1,094, 956
+//   FP8    8 rows 721, 979; 16: 846, 1,005; 24: 1,055, 1,018; 48: 1,301, 1,042; 64: 1,420, 1,081
+//   8 active rows in a launch for 64: BF16 610, 782; FP8 759, 959
+// The line is where a full BF16 batch has lost 5%.  A full FP8 batch loses
+// from about 24 rows on; one whose streams have ended down to 16 gains 15%.
 enum DecPro { DPRO_TMA = 0, DPRO_RMS = 1, DPRO_FP8 = 2 };   // operand: by TMA, RMSNorm of x, E4M3 of x
-constexpr int kPlainVecs = 12;              // DPRO_FP8: float4 values of a row per lane (1,536 columns)
+constexpr int kPlainVecs = 12;              // DPRO_FP8: float4 values of a row per lane (1,536 columns, the
+                                            // full model's widest row; wider rows take the row kernels)
 constexpr int kDecSmemMax = 227 * 1024;
 constexpr int kDecMaxRows = 64;
 struct TcDec {

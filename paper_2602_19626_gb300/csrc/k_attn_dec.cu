@@ -26,7 +26,6 @@
 // position rotates its k, rounds k and v to BF16 and puts them into the ring
 // and into its tiles.
 //
-//
 // Measured (GB300, full model, nc_decode, time per token step, with the pair
 // tiles and the partials merged through global memory -> this kernel): one
 // BF16 stream of 300 tokens 703 -> 556 us; 48 FP8 streams of up to 160 tokens

@@ -1,10 +1,9 @@
 // tcgen05 projections of a decode step: few rows, so the kernel is bound by
 // latency, not by bytes or products.
 //
-// Y[n][m] = sum_k W[m][k] X[n][k] as in k_gemm_tc.cu, with the same MMA
-// shape over K (128 weight rows, K blocks of 128 bytes, four instructions
-// each, in order), so every output element has the same bits.  What differs
-// is everything around the products:
+// Y[n][m] = sum_k W[m][k] X[n][k] as in k_gemm_tc.cu, with the same steps over
+// K (blocks of 128 bytes, four instructions each, in order), so every output
+// element has the same bits.  What differs is everything around the products:
 //   - a CTA stores kDecM = 32 weight rows instead of 128, so a 576-row
 //     projection spreads over 18 SMs instead of 5 and its weights arrive in a
 //     quarter of the time.  The MMA takes M = 64 (the products are those of
@@ -55,7 +54,7 @@ struct Pick {
 };
 
 // Bytes after the barriers' 1024: the weights' blocks, the operand's, and
-// what the MMA's 128 rows read past the last weight block.
+// what the MMA's 64 rows read past the last weight block.
 __host__ __device__ inline size_t dec_smem_bytes(int nk, int bn) {
   const size_t a = (size_t)nk * kABlk, b = (size_t)nk * bn * kBlkBytes;
   const size_t over = (size_t)(nk - 1) * kABlk + (size_t)kMmaM * kBlkBytes;   // end of the last block's read
@@ -275,9 +274,16 @@ cudaError_t dec_prepare_t() {
                               kDecSmemMax);
 }
 
-// The variants of a row-making prologue: one row per warp up to 8 rows; 16
-// warps of two rows at a time for more, in tiles of 32 or (above 32 rows) 64
-// rows, so that the CTAs stay within one wave.
+// The variants of a row-making prologue: one row per warp and 8 warps up to 8
+// rows; 16 warps of two rows at a time for more, in tiles of 32 or (above 32
+// rows) 64 rows.  Measured (GB300, full model, one nc_step_probe, in us):
+//   8 warps, then 16 warps of two rows: BF16 8 rows 551, 599; 16: 636, 661;
+//   24: 697, 686; 32: 762, 710; FP8 8 rows 722, 759; 16: 871, 845
+//   above 32 rows 64-row tiles, then 32-row tiles of 16 and of 8 warps: BF16
+//   48 rows 849, 871, 796; 64: 905, 934, 859; 32 active rows in a launch for
+//   64: 721, 722, 771
+// The E4M3 rows of a residual projection, 8 warps, then 16: 8 rows 722, 723;
+// 16: 981, 871.
 template <typename F>
 cudaError_t dec_rms(int kind_bf16, int epi, F f) {
   if (epi == EPI_STORE) return kind_bf16 ? f(Pick<1, EPI_STORE>()) : f(Pick<0, EPI_STORE>());

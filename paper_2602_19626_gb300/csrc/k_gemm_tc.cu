@@ -465,7 +465,9 @@ __device__ void write_operand(const float* buf, int cols, int j, void* out, floa
 
 // The same for rows of at most 32 kRowVals columns: a warp per row (the sums
 // in the order of the 256-thread row), eight rows per CTA, no block barrier.
-// Measured for 3,072 rows of 576: 8.9 us a launch with a CTA per row.
+// Measured (GB300, 4,096 rows of 576, gate/up projection with its operand):
+// 36.0 us, 41.1 with a CTA per row; the E4M3 operand alone likewise (down
+// projection with its operand 22.1 us, 27.8).
 template <int KB>
 __global__ void __launch_bounds__(256) k_act_rmsnorm_w(Batch b, const float* x, const float* gain, int cols, float eps,
                                                        void* out, float* out_scale) {

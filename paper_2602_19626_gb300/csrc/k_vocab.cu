@@ -3,14 +3,12 @@
 // prefix sum (Sec. 3.3), the head / mixer updates, and the N-gram tables.
 //
 // One stream is handled by a cluster of CTAs (8 or 16 for the per-token
-// step, kVocabCluster for the standalone quantiser); each CTA owns a
-// contiguous chunk of the vocabulary and each thread a contiguous run of E
-// symbols.  The standalone quantiser reduces thread -> warp (fixed xor tree)
-// -> CTA (warps in order) -> cluster (ranks in order through distributed
-// shared memory); the per-token step goes thread -> warp -> every CTA's inbox
-// (one cluster barrier in the step kernel, one exchange round on each CTA's
-// mbarrier in the prefill loop) -> the same fixed reduction in every warp.
-// Every result is independent of the batch, the slot and the launch.
+// step, kP2cCtas = 4 for a row of the standalone quantiser); each CTA owns a
+// contiguous chunk of the vocabulary.  A reduction goes thread -> warp ->
+// every CTA's inbox (one cluster barrier in the step kernel and the quantiser,
+// one exchange round on each CTA's mbarrier in the prefill loop) -> the same
+// fixed reduction in every warp.  The mixed NLL takes a CTA per row.  Every
+// result is independent of the batch, the slot and the launch.
 #include <algorithm>
 
 #include <cooperative_groups.h>
@@ -663,9 +661,8 @@ __device__ void ng_snapshot(const Dims& D, const StreamDev& st, NgSnap* out, int
 // or the coder interval of the observed token) and / or update (head and
 // mixer, then the N-gram and the stream's bookkeeping).  A caller with its
 // own coder runs the two in separate launches; the decoder gives the coder's
-// target and takes both in one (predict, a search of the CDF in memory and an
-// update that made the softmax again took 26 us a token for one stream, 73 us
-// for 48); the arithmetic is the same in every case.
+// target and takes both in one, with the token's search on the counts in
+// registers between them; the arithmetic is the same in every case.
 template <int E, bool FULL, int CL>
 __global__ void __launch_bounds__(step_threads<CL>(), 1) k_vocab(Dims D, Batch b, VocabIO io) {
   extern __shared__ float4 dyn4[];
@@ -1682,9 +1679,9 @@ __global__ void k_prepare_prefill(Batch b, int n_streams, int m, int V, const in
 // then each warp scans its own pieces.  A row of the CDF has V + 1 entries, so
 // rows start at any of the four offsets of a 16-byte vector: lanes pass their
 // last entries on and store aligned vectors.
-// Bound by memory.  The first version (eight CTAs of 512 threads, 12
-// consecutive symbols per thread, block and cluster rounds of 64-bit shuffles
-// and three cluster barriers) took 117 us for 256 rows of 49,152 (100 MB).
+// Bound by memory: 33 us for 256 rows of 49,152 (101 MB; 117 us with eight CTAs
+// of 512 threads, 12 consecutive symbols per thread and three cluster
+// barriers).  A call of one row takes 34 us either way, launch and status copy.
 constexpr int kP2cCtas = 4, kP2cThreads = 256;
 constexpr int kP2cWarps = kP2cCtas * kP2cThreads / 32;     // 32: one inbox entry per lane
 struct P2cPart {
@@ -2136,7 +2133,9 @@ cudaError_t launch_prepare_prefill(const Batch& b, int n_streams, int m, int V, 
 
 cudaError_t launch_probs_to_cdf(const float* p, int n, int V, int log2T, uint32_t floor_c, uint32_t* cdf,
                                 int32_t* status, bool per_row, cudaStream_t s) {
-  // pieces of 128 symbols per warp, in powers of two but for the full vocabulary's 12
+  // pieces of 128 symbols per warp, in powers of two, and 12: with its 80
+  // registers three CTAs of 256 threads share an SM, with the 145 of 16 pieces
+  // one has it (a call of 256 rows of 49,152 takes 61 us, with 16 pieces 109)
   const int it = (V + 128 * kP2cWarps - 1) / (128 * kP2cWarps);
   auto go = [&](auto kern) {
     kern<<<n * kP2cCtas, kP2cThreads, 0, s>>>(p, V, log2T, floor_c, cdf, status, per_row);

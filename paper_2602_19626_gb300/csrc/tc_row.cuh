@@ -35,7 +35,8 @@ __device__ __forceinline__ void swiglu_pair(bool mine, int M, float* h_out, void
 
 // A row of up to 32 kRowVals columns over one warp, column lane + 32 i in
 // value i.
-constexpr int kRowVals = 20;                 // 640 columns: 576 in whole 128-byte E4M3 blocks
+constexpr int kRowVals = 20;                 // 640 columns: the full model's 576 in whole 128-byte E4M3
+                                             // blocks; wider rows take the kernels of a CTA per row
 
 __device__ __forceinline__ void load_row(const float* xr, int cols, int lane, float (&x)[kRowVals]) {
 #pragma unroll
