@@ -2393,7 +2393,7 @@ extern "C" int nc_gemm_tc(const void* W, const void* X, const float* w_scale, co
   g.x_scale = x_scale;
   g.y = Y;
   g.status = w.p;
-  cudaError_t el = prepare_gemm_store(g);
+  cudaError_t el = prepare_gemm_store(g, dev);
   if (el == cudaSuccess) el = launch_gemm_tc(g, EPI_STORE, s, false);
   int32_t gave_up = 0;
   const cudaError_t ef = w.finish(s, &gave_up);

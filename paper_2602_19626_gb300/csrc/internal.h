@@ -77,6 +77,7 @@ constexpr int kTmapBytes = 128;             // one CUtensorMap
 
 struct Dims {
   int pdl;                  // launch step kernels with programmatic dependent launch
+  int cl16;                 // clusters of 16 CTAs of the vocabulary kernels can be placed on the device
   const float2* rope_tab;   // [kRopeLevels][256][32]
   int n_layers, d, hq, hkv, F, V, L, C;
   int qkv_rows;             // (hq + 2 hkv) * 64
@@ -84,7 +85,6 @@ struct Dims {
   int kv_bf16;              // 1: KV cache in BF16
   int attn_cluster;         // CTAs per (stream, KV head) in the FP32-cache attention: 1, 2, 4 or 8; 0 = by batch size
   int n_sm;                 // SMs of the device
-  int cl16;                 // clusters of 16 CTAs of the vocabulary kernels can be placed on it
   int order;                // N-gram order (0 = off)
   int skip;                 // confidence skip: p = p_ng when H(p_ng) < kSkipBits
   int use_head;
@@ -382,7 +382,8 @@ cudaError_t launch_act_plain(const Dims& D, const Batch& b, const float* x, int 
 cudaError_t prepare_model_kernels(const Dims& D, int fmt);
 cudaError_t prepare_vocab_kernels(Dims* D);       // sets D->cl16
 cudaError_t prepare_tc_kernels();
-cudaError_t prepare_gemm_store(const TcGemm& g);   // of the variant that launch_gemm_tc(g, EPI_STORE) takes
+// The variant that launch_gemm_tc(g, EPI_STORE) takes on the current device `dev`.
+cudaError_t prepare_gemm_store(const TcGemm& g, int dev);
 
 // status: a word per row (per_row), or one word that any bad row raises.
 cudaError_t launch_probs_to_cdf(const float* p, int n, int V, int log2T, uint32_t floor,

@@ -17,6 +17,8 @@
 // frees its tensor memory and exits it waits, with the same bound, for what it
 // already issued: the products (one commit after the last one issued) and the
 // TMA loads no product consumed, so nothing lands in a CTA that has exited.
+#include <atomic>
+
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
@@ -351,14 +353,20 @@ cudaError_t tc_pick(const TcGemm& g, F f) {
   return cudaErrorInvalidValue;
 }
 
-// The shared-memory limit of the variant g asks for, in the current device's
-// context (a limit holds for one context).
+// The shared-memory limit of the variant g asks for, on the current device.
+// dev >= 0 (that device): not again where this call has set it, a bit per
+// device and variant (set each time it takes 0.7 of a small nc_gemm_tc's 30 us).
 template <int KB, int EPI>
-cudaError_t prepare_tc_one(const TcGemm& g) {
-  return tc_pick<KB>(g, [](auto t) {
+cudaError_t prepare_tc_one(const TcGemm& g, int dev = -1) {
+  return tc_pick<KB>(g, [dev](auto t) {
     using T = decltype(t);
-    return cudaFuncSetAttribute(k_gemm_tc<T::BN, T::STAGES, KB, EPI, T::KP, T::OCC>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem);
+    static std::atomic<unsigned long long> set{0};
+    const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0;
+    if (set.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(k_gemm_tc<T::BN, T::STAGES, KB, EPI, T::KP, T::OCC>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem);
+    if (e == cudaSuccess) set.fetch_or(bit, std::memory_order_release);
+    return e;
   });
 }
 
@@ -587,8 +595,8 @@ cudaError_t prepare_tc_kernels() {
   return e;
 }
 
-cudaError_t prepare_gemm_store(const TcGemm& g) {
-  return g.kind_bf16 ? prepare_tc_one<1, EPI_STORE>(g) : prepare_tc_one<0, EPI_STORE>(g);
+cudaError_t prepare_gemm_store(const TcGemm& g, int dev) {
+  return g.kind_bf16 ? prepare_tc_one<1, EPI_STORE>(g, dev) : prepare_tc_one<0, EPI_STORE>(g, dev);
 }
 
 cudaError_t launch_gemm_tc(const TcGemm& g, int epi, cudaStream_t s, bool pdl) {
